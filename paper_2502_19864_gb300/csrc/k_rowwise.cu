@@ -1,12 +1,13 @@
-// k_rowwise.cu -- row-wise fused kernels of the step: adapters (Eq. 1) fused with the
-// residual add and the block's normalisation, the adapter backward with its in-kernel
-// deterministic weight-gradient reduction, LayerNorm / RMSNorm, the heads and their
+// k_rowwise.cu -- row-wise fused kernels of the step: the adapters' dispatch (Eq. 1) and the
+// fixed-order sum of their weight-gradient partials, LayerNorm / RMSNorm, the heads and their
 // cross-entropy, and Adam.
 #include "common.cuh"
 #include "kernels.h"
 
 namespace ra {
 namespace {
+
+constexpr int MAXM = 128;          // adapter bottleneck upper bound
 
 template <typename T>
 __device__ __forceinline__ float ldf(const void* p, int64_t i) {
@@ -15,275 +16,6 @@ __device__ __forceinline__ float ldf(const void* p, int64_t i) {
 template <typename T>
 __device__ __forceinline__ void stf(void* p, int64_t i, float v) {
   reinterpret_cast<T*>(p)[i] = from_f<T>(v);
-}
-
-constexpr int WARPS = 8;
-constexpr int RPW = 2;             // rows per warp in the adapter row kernels
-constexpr int ROWS = WARPS * RPW;  // rows per CTA
-constexpr int MAXM = 128;          // adapter bottleneck upper bound
-constexpr int MC = MAXM / 32;      // bottleneck columns per lane
-
-// ---------------------------------------------------------------------------------------
-// Adapter forward (Eq. 1) + residual + norm.  Warp w owns rows (blockIdx*ROWS + w*RPW + r).
-// smem: rows [ROWS][H] f32 (adapter input, then the pre-norm sum), s [ROWS][m] f32.
-// ---------------------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(WARPS * 32) adapter_fwd_kernel(AdapterFwdArgs a) {
-  extern __shared__ float sm[];
-  const int H = a.H, m = a.m;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float* rows = sm + (size_t)warp * RPW * H;
-  float* sv = sm + (size_t)ROWS * H + warp * RPW * MAXM;
-  const int t0 = blockIdx.x * ROWS + warp * RPW;
-
-  for (int r = 0; r < RPW; ++r) {
-    int t = t0 + r;
-    for (int i = lane; i < H; i += 32) rows[r * H + i] = t < a.T ? ldf<T>(a.a, (int64_t)t * H + i) : 0.f;
-  }
-  __syncwarp();
-  // z = a W_down  (lanes over bottleneck columns j = lane + 32c)
-  float z[RPW][MC];
-#pragma unroll
-  for (int r = 0; r < RPW; ++r)
-#pragma unroll
-    for (int c = 0; c < MC; ++c) z[r][c] = 0.f;
-  for (int i = 0; i < H; ++i) {
-    float w[MC];
-#pragma unroll
-    for (int c = 0; c < MC; ++c) {
-      int j = lane + 32 * c;
-      w[c] = j < m ? a.Wd[(int64_t)i * m + j] : 0.f;
-    }
-#pragma unroll
-    for (int r = 0; r < RPW; ++r) {
-      float x = rows[r * H + i];
-#pragma unroll
-      for (int c = 0; c < MC; ++c) z[r][c] = fmaf(x, w[c], z[r][c]);
-    }
-  }
-#pragma unroll
-  for (int r = 0; r < RPW; ++r) {
-    int t = t0 + r;
-#pragma unroll
-    for (int c = 0; c < MC; ++c) {
-      int j = lane + 32 * c;
-      if (j < m) {
-        sv[r * MAXM + j] = gelu_f(z[r][c]);
-        if (a.z && t < a.T) a.z[(int64_t)t * m + j] = z[r][c];
-      }
-    }
-  }
-  __syncwarp();
-  // out = a + GELU(z) W_up, in chunks of 256 columns (lanes over i = i0 + lane + 32cc)
-  for (int i0 = 0; i0 < H; i0 += 256) {
-    float acc[RPW][8];
-#pragma unroll
-    for (int r = 0; r < RPW; ++r)
-#pragma unroll
-      for (int cc = 0; cc < 8; ++cc) acc[r][cc] = 0.f;
-    for (int j = 0; j < m; ++j) {
-      float w[8];
-#pragma unroll
-      for (int cc = 0; cc < 8; ++cc) {
-        int i = i0 + lane + 32 * cc;
-        w[cc] = i < H ? a.Wu[(int64_t)j * H + i] : 0.f;
-      }
-#pragma unroll
-      for (int r = 0; r < RPW; ++r) {
-        float s = sv[r * MAXM + j];
-#pragma unroll
-        for (int cc = 0; cc < 8; ++cc) acc[r][cc] = fmaf(s, w[cc], acc[r][cc]);
-      }
-    }
-#pragma unroll
-    for (int r = 0; r < RPW; ++r) {
-      int t = t0 + r;
-#pragma unroll
-      for (int cc = 0; cc < 8; ++cc) {
-        int i = i0 + lane + 32 * cc;
-        if (i < H) {
-          float res = 0.f;
-          if (t < a.T && a.resid)
-            res = a.decoder ? reinterpret_cast<const float*>(a.resid)[(int64_t)t * H + i]
-                            : ldf<T>(a.resid, (int64_t)t * H + i);
-          rows[r * H + i] = res + rows[r * H + i] + acc[r][cc];
-        }
-      }
-    }
-  }
-  __syncwarp();
-  // normalisation of the residual sum
-  for (int r = 0; r < RPW; ++r) {
-    int t = t0 + r;
-    if (t >= a.T) break;
-    float* v = rows + r * H;
-    if (a.no_norm) {
-      for (int i = lane; i < H; i += 32) stf<T>(a.y, (int64_t)t * H + i, v[i]);
-    } else if (!a.decoder) {
-      float s = 0.f;
-      for (int i = lane; i < H; i += 32) s += v[i];
-      float mu = warp_sum(s) / H;
-      float q = 0.f;
-      for (int i = lane; i < H; i += 32) { float d = v[i] - mu; q += d * d; }
-      float rstd = rsqrtf(warp_sum(q) / H + a.eps);
-      for (int i = lane; i < H; i += 32) {
-        float xh = (v[i] - mu) * rstd;
-        stf<T>(a.y, (int64_t)t * H + i, xh * a.gamma[i] + a.beta[i]);
-        if (a.xhat) stf<T>(a.xhat, (int64_t)t * H + i, xh);
-      }
-      if (a.rstd && lane == 0) a.rstd[t] = rstd;
-    } else {
-      float q = 0.f;
-      for (int i = lane; i < H; i += 32) q += v[i] * v[i];
-      float rstd = rsqrtf(warp_sum(q) / H + a.eps);
-      for (int i = lane; i < H; i += 32) {
-        a.x_out[(int64_t)t * H + i] = v[i];
-        stf<T>(a.y, (int64_t)t * H + i, v[i] * rstd * a.gamma[i]);
-      }
-      if (a.rstd && lane == 0) a.rstd[t] = rstd;
-    }
-  }
-}
-
-// ---------------------------------------------------------------------------------------
-// Adapter backward, row part: dz = (g W_up^T) * GELU'(z), dh = g + dz W_down^T
-// ---------------------------------------------------------------------------------------
-template <typename TO>
-__global__ void __launch_bounds__(WARPS * 32) adapter_bwd_rows_kernel(AdapterBwdArgs a) {
-  extern __shared__ float sm[];
-  const int H = a.H, m = a.m;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float* rows = sm + (size_t)warp * RPW * H;
-  float* dzs = sm + (size_t)ROWS * H + warp * RPW * MAXM;
-  const int t0 = blockIdx.x * ROWS + warp * RPW;
-  for (int r = 0; r < RPW; ++r) {
-    int t = t0 + r;
-    for (int i = lane; i < H; i += 32) rows[r * H + i] = t < a.T ? a.g[(int64_t)t * H + i] : 0.f;
-  }
-  __syncwarp();
-  float ds[RPW][MC];
-#pragma unroll
-  for (int r = 0; r < RPW; ++r)
-#pragma unroll
-    for (int c = 0; c < MC; ++c) ds[r][c] = 0.f;
-  for (int i = 0; i < H; ++i) {
-    float w[MC];
-#pragma unroll
-    for (int c = 0; c < MC; ++c) {
-      int j = lane + 32 * c;
-      w[c] = j < m ? a.WuT[(int64_t)i * m + j] : 0.f;
-    }
-#pragma unroll
-    for (int r = 0; r < RPW; ++r) {
-      float x = rows[r * H + i];
-#pragma unroll
-      for (int c = 0; c < MC; ++c) ds[r][c] = fmaf(x, w[c], ds[r][c]);
-    }
-  }
-#pragma unroll
-  for (int r = 0; r < RPW; ++r) {
-    int t = t0 + r;
-#pragma unroll
-    for (int c = 0; c < MC; ++c) {
-      int j = lane + 32 * c;
-      if (j < m) {
-        float dz = 0.f;
-        if (t < a.T) {
-          dz = ds[r][c] * gelu_grad_f(a.z[(int64_t)t * m + j]);
-          a.dz[(int64_t)t * m + j] = dz;
-        }
-        dzs[r * MAXM + j] = dz;
-      }
-    }
-  }
-  __syncwarp();
-  if (!a.dh) return;
-  for (int i0 = 0; i0 < H; i0 += 256) {
-    float acc[RPW][8];
-#pragma unroll
-    for (int r = 0; r < RPW; ++r)
-#pragma unroll
-      for (int cc = 0; cc < 8; ++cc) acc[r][cc] = 0.f;
-    for (int j = 0; j < m; ++j) {
-      float w[8];
-#pragma unroll
-      for (int cc = 0; cc < 8; ++cc) {
-        int i = i0 + lane + 32 * cc;
-        w[cc] = i < H ? a.WdT[(int64_t)j * H + i] : 0.f;
-      }
-#pragma unroll
-      for (int r = 0; r < RPW; ++r) {
-        float d = dzs[r * MAXM + j];
-#pragma unroll
-        for (int cc = 0; cc < 8; ++cc) acc[r][cc] = fmaf(d, w[cc], acc[r][cc]);
-      }
-    }
-#pragma unroll
-    for (int r = 0; r < RPW; ++r) {
-      int t = t0 + r;
-      if (t >= a.T) continue;
-#pragma unroll
-      for (int cc = 0; cc < 8; ++cc) {
-        int i = i0 + lane + 32 * cc;
-        if (i < H) stf<TO>(a.dh, (int64_t)t * H + i, rows[r * H + i] + acc[r][cc]);
-      }
-    }
-  }
-}
-
-// Weight-gradient partials over a chunk of rows:
-//   pWu[c][j][i]  = sum_{t in chunk c} GELU(z[t, j]) g[t, i]          (dW_up  = GELU(z)^T g)
-//   pWdT[c][j][i] = sum_{t in chunk c} h[t, i] dz[t, j]                (dW_down^T = dz^T h)
-// CTA: 64 columns i x all m; thread owns i = tid % 64, j = tid/64 + 4c.
-constexpr int DW_COLS = 64, DW_ROWS = 16;
-template <typename T>
-__global__ void __launch_bounds__(256) adapter_dw_partial_kernel(AdapterBwdArgs a, int chunk) {
-  __shared__ float gS[DW_ROWS][DW_COLS], hS[DW_ROWS][DW_COLS];
-  __shared__ float sS[DW_ROWS][MAXM], dzS[DW_ROWS][MAXM];
-  const int H = a.H, m = a.m;
-  const int i0 = blockIdx.x * DW_COLS, c = blockIdx.y;
-  const int tid = threadIdx.x, il = tid % DW_COLS, jg = tid / DW_COLS;
-  const int tb = c * chunk, te = min(a.T, tb + chunk);
-  float aWu[MAXM / 4], aWd[MAXM / 4];
-#pragma unroll
-  for (int q = 0; q < MAXM / 4; ++q) { aWu[q] = 0.f; aWd[q] = 0.f; }
-  for (int t0 = tb; t0 < te; t0 += DW_ROWS) {
-    __syncthreads();
-    for (int e = tid; e < DW_ROWS * DW_COLS; e += 256) {
-      int r = e / DW_COLS, i = e % DW_COLS, t = t0 + r;
-      bool in = t < te && i0 + i < H;
-      gS[r][i] = in ? a.g[(int64_t)t * H + i0 + i] : 0.f;
-      hS[r][i] = in ? ldf<T>(a.h, (int64_t)t * H + i0 + i) : 0.f;
-    }
-    for (int e = tid; e < DW_ROWS * MAXM; e += 256) {
-      int r = e / MAXM, j = e % MAXM, t = t0 + r;
-      bool in = t < te && j < m;
-      sS[r][j] = in ? gelu_f(a.z[(int64_t)t * m + j]) : 0.f;
-      dzS[r][j] = in ? a.dz[(int64_t)t * m + j] : 0.f;
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int r = 0; r < DW_ROWS; ++r) {
-      float gv = gS[r][il], hv = hS[r][il];
-#pragma unroll
-      for (int q = 0; q < MAXM / 4; ++q) {
-        int j = jg + 4 * q;
-        aWu[q] = fmaf(sS[r][j], gv, aWu[q]);
-        aWd[q] = fmaf(dzS[r][j], hv, aWd[q]);
-      }
-    }
-  }
-  if (i0 + il >= H) return;
-  float* pWu = a.partials + (size_t)c * 2 * H * m;
-  float* pWdT = pWu + (size_t)H * m;
-#pragma unroll
-  for (int q = 0; q < MAXM / 4; ++q) {
-    int j = jg + 4 * q;
-    if (j < m) {
-      pWu[(size_t)j * H + i0 + il] = aWu[q];
-      pWdT[(size_t)j * H + i0 + il] = aWd[q];
-    }
-  }
 }
 
 // Fixed-order sum of the partials: dW_up[j][i] and dW_down[i][j].
@@ -318,6 +50,7 @@ __global__ void adapter_dw_reduce_kernel(const float* partials, int nchunk, int 
 // Chunk count of the weight-gradient reduction: a pure function of (T, H), so the scratch
 // size planned on the host and the grid launched on any device agree, and the reduction
 // order (hence the bits of the result) does not depend on the device.
+constexpr int DW_COLS = 64, DW_ROWS = 16;
 constexpr int kDwTargetCtas = 304;
 int dw_chunks(int T, int H) {
   int colblocks = (H + DW_COLS - 1) / DW_COLS;
@@ -1132,17 +865,7 @@ cudaError_t adapter_fwd(const AdapterFwdArgs& a, cudaStream_t st) {
   if (a.m > MAXM || a.m <= 0) return cudaErrorInvalidValue;
   if (a.dtype == DT_BF16 && a.WdT_b && a.WuT_b && adapter_mma_ok(a.H, a.m))
     return adapter_fwd_mma(a, a.WdT_b, a.WuT_b, st);
-  size_t smem = ((size_t)ROWS * a.H + ROWS * MAXM) * sizeof(float);
-  unsigned grid = blocks_for(a.T, ROWS);
-  if (a.dtype == DT_BF16) {
-    cudaFuncSetAttribute(adapter_fwd_kernel<bf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    adapter_fwd_kernel<bf16><<<grid, WARPS * 32, smem, st>>>(a);
-  } else {
-    cudaFuncSetAttribute(adapter_fwd_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    adapter_fwd_kernel<float><<<grid, WARPS * 32, smem, st>>>(a);
-  }
-  note_launch(1);
-  return cudaGetLastError();
+  return adapter_fwd_simt(a, st);
 }
 
 size_t adapter_bwd_partials_floats(int T, int H, int m) {
@@ -1165,28 +888,7 @@ cudaError_t adapter_bwd(const AdapterBwdArgs& a, cudaStream_t st) {
   // never changes which kernels compute dz and dW
   if (a.dtype == DT_BF16 && a.Wu_b && a.Wd_b && adapter_mma_ok(a.H, a.m))
     return adapter_bwd_mma(a, a.Wu_b, a.Wd_b, st);
-  size_t smem = ((size_t)ROWS * a.H + ROWS * MAXM) * sizeof(float);
-  unsigned grid = blocks_for(a.T, ROWS);
-  if (a.dh_dtype == DT_BF16) {
-    cudaFuncSetAttribute(adapter_bwd_rows_kernel<bf16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    adapter_bwd_rows_kernel<bf16><<<grid, WARPS * 32, smem, st>>>(a);
-  } else {
-    cudaFuncSetAttribute(adapter_bwd_rows_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    adapter_bwd_rows_kernel<float><<<grid, WARPS * 32, smem, st>>>(a);
-  }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  int nchunk = dw_chunks(a.T, a.H);
-  int chunk = (a.T + nchunk - 1) / nchunk;
-  dim3 g2((a.H + DW_COLS - 1) / DW_COLS, nchunk);
-  if (a.dtype == DT_BF16) adapter_dw_partial_kernel<bf16><<<g2, 256, 0, st>>>(a, chunk);
-  else adapter_dw_partial_kernel<float><<<g2, 256, 0, st>>>(a, chunk);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  int64_t n = 2LL * a.H * a.m;
-  (void)launch_pdl(adapter_dw_reduce_kernel, dim3(blocks_for(n, 256)), dim3(256), (size_t)0, st, a.partials, nchunk, a.H, a.m, a.dWd, a.dWu);
-  note_launch(3);
-  return cudaGetLastError();
+  return adapter_bwd_simt(a, st);
 }
 
 cudaError_t layernorm_bwd(const float* dy, const float* dy2, const void* xhat, const float* rstd,

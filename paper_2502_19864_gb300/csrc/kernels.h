@@ -172,6 +172,7 @@ struct AdapterFwdArgs {
 cudaError_t adapter_fwd(const AdapterFwdArgs& a, cudaStream_t st);
 cudaError_t adapter_fwd_mma(const AdapterFwdArgs& a, const void* WdT_b, const void* WuT_b,
                             cudaStream_t st);
+cudaError_t adapter_fwd_simt(const AdapterFwdArgs& a, cudaStream_t st);
 bool adapter_mma_ok(int H, int m);
 
 // Adapter backward, row part: dz = (g Wu^T) * GELU'(z) -> dz (f32 [T, m]);
@@ -197,6 +198,7 @@ size_t adapter_bwd_partials_floats(int T, int H, int m);
 cudaError_t adapter_bwd(const AdapterBwdArgs& a, cudaStream_t st);
 cudaError_t adapter_bwd_mma(const AdapterBwdArgs& a, const void* Wu_b, const void* Wd_b,
                             cudaStream_t st);
+cudaError_t adapter_bwd_simt(const AdapterBwdArgs& a, cudaStream_t st);
 // chunk count of the dW reduction (a pure function of T and H) and its fixed-order sum
 int adapter_dw_chunks(int T, int H);
 cudaError_t adapter_dw_reduce(const float* partials, int nchunk, int H, int m, float* dWd,
