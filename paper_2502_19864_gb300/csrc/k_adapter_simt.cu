@@ -24,6 +24,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "simt.cuh"
 
 namespace ra {
 namespace {
@@ -36,13 +37,6 @@ __device__ __forceinline__ float4 ld4v(const T* p);
 template <>
 __device__ __forceinline__ float4 ld4v<float>(const float* p) {
   return __ldg(reinterpret_cast<const float4*>(p));
-}
-__device__ __forceinline__ float4 ld4s(const float* p) { return *reinterpret_cast<const float4*>(p); }
-__device__ __forceinline__ float4 ld4s(const bf16* p) {
-  const uint2 u = *reinterpret_cast<const uint2*>(p);
-  const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.x));
-  const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.y));
-  return make_float4(a.x, a.y, b.x, b.y);
 }
 template <>
 __device__ __forceinline__ float4 ld4v<bf16>(const bf16* p) {
@@ -78,37 +72,6 @@ __device__ __forceinline__ void st4(T* row, int c, int n, bool vec, float4 v) {
   if (c + 1 < n) row[c + 1] = from_f<T>(v.y);
   if (c + 2 < n) row[c + 2] = from_f<T>(v.z);
   if (c + 3 < n) row[c + 3] = from_f<T>(v.w);
-}
-
-// ---- per-warp copy pipeline: chunks of 8 k (phase 1: X [R][8] and W [8][MP]; phase 2: W' [8][32]),
-// NS deep; cp.async where the operand rows allow 16-byte copies, plain stores else
-__device__ __forceinline__ void cp16(void* dst, const void* src, bool valid) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
-               "l"(src), "r"(valid ? 16 : 0)
-               : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-// nr x nc block of a row-major matrix (row stride ld, nc a multiple of 4) at src into dst (row stride
-// ldd): entry (r, c) is taken where r < vr and c < vc and zero elsewhere.  All lanes of a warp.
-template <typename T>
-__device__ __forceinline__ void copy_block(T* dst, int ldd, const T* src, size_t ld, int nr, int nc, int vr, int vc,
-                                           bool vec, int lane) {
-  constexpr int E = 16 / sizeof(T);
-  if (vec) {
-    const int per = nc / E;
-    for (int e = lane; e < nr * per; e += 32) {
-      const int r = e / per, c = (e % per) * E;
-      const bool ok = r < vr && c < vc;
-      cp16(dst + r * ldd + c, src + (ok ? r * ld + c : 0), ok);
-    }
-  } else {
-    for (int e = lane; e < nr * nc; e += 32) {
-      const int r = e / nc, c = e % nc;
-      dst[r * ldd + c] = r < vr && c < vc ? src[r * ld + c] : from_f<T>(0.f);
-    }
-  }
 }
 
 // Shared memory (bytes): [0, s) first the warps' copy rings, then the phase 1 partials [NW][R][MP], then

@@ -5,11 +5,13 @@
 // meet a 1e-4 relative bar) and of shapes the tensor-core kernel does not take.
 #include "common.cuh"
 #include "kernels.h"
+#include "simt.cuh"
 
 namespace ra {
 namespace {
 
-constexpr int BM = 64, BN = 64, BK = 16, NT = 256;
+// 32 x 32 output tiles; the 8 warps of a CTA split K
+constexpr int BT = 32, NW = 8, NT = NW * 32, KC = 8, NS = 3, LDP = BT + 8;
 
 template <typename T>
 __device__ __forceinline__ float ld(const void* p, int64_t i) {
@@ -61,62 +63,167 @@ __device__ __forceinline__ void epilogue(const GemmArgs& g, int m, int n, float 
   }
 }
 
-template <typename TI>
-__global__ void __launch_bounds__(NT) gemm_simt_kernel(GemmArgs g) {
-  __shared__ float As[BK][BM + 4];
-  __shared__ float Bs[BK][BN + 4];
-  const int tid = threadIdx.x;
-  const int tx = tid & 15, ty = tid >> 4;
-  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+// four consecutive values of a row (n a multiple of 4, `vec`: 16-byte (f32) or 8-byte (bf16) accesses)
+__device__ __forceinline__ float4 ld4_dt(const void* p, int dt, int64_t i, bool vec) {
+  if (!vec) return make_float4(ld_dt(p, dt, i), ld_dt(p, dt, i + 1), ld_dt(p, dt, i + 2), ld_dt(p, dt, i + 3));
+  if (dt == DT_F32) return *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(p) + i);
+  return ld4s(reinterpret_cast<const bf16*>(p) + i);
+}
+__device__ __forceinline__ void st4_dt(void* p, int dt, int64_t i, bool vec, float4 v) {
+  if (!vec) {
+    st_dt(p, dt, i, v.x); st_dt(p, dt, i + 1, v.y); st_dt(p, dt, i + 2, v.z); st_dt(p, dt, i + 3, v.w);
+  } else if (dt == DT_F32) {
+    *reinterpret_cast<float4*>(reinterpret_cast<float*>(p) + i) = v;
+  } else {
+    __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
+    *reinterpret_cast<uint2*>(reinterpret_cast<bf16*>(p) + i) = make_uint2(*reinterpret_cast<uint32_t*>(&a), *reinterpret_cast<uint32_t*>(&b));
+  }
+}
+// the epilogue of columns n .. n + 3, all below N
+__device__ __forceinline__ void epilogue4(const GemmArgs& g, int m, int n, float4 u, bool vec) {
+  const int64_t c = (int64_t)m * g.ldc + n;
+  if (g.bias && g.epi != EPI_MUL && g.epi != EPI_RESID && g.epi != EPI_DSWIGLU) {
+    u.x += g.bias[n]; u.y += g.bias[n + 1]; u.z += g.bias[n + 2]; u.w += g.bias[n + 3];
+  }
+  if (g.epi == EPI_BIAS_GELU || g.epi == EPI_BIAS_GELU_G) {
+    if (g.C)
+      st4_dt(g.C, g.c_dtype, c, vec,
+             g.epi == EPI_BIAS_GELU ? u : make_float4(gelu_grad_f(u.x), gelu_grad_f(u.y), gelu_grad_f(u.z), gelu_grad_f(u.w)));
+    st4_dt(g.C2, g.c2_dtype, (int64_t)m * g.ldc2 + n, vec, make_float4(gelu_f(u.x), gelu_f(u.y), gelu_f(u.z), gelu_f(u.w)));
+    return;
+  }
+  if (g.epi == EPI_DSWIGLU) {
+    const int64_t gc = gate_col(n), ax = (int64_t)m * g.ldaux + gc, cc = (int64_t)m * g.ldc + gc;
+    const float4 gt = ld4_dt(g.aux, g.aux_dtype, ax, vec), up = ld4_dt(g.aux, g.aux_dtype, ax + 64, vec);
+    st4_dt(g.C, g.c_dtype, cc, vec, make_float4(u.x * up.x * silu_grad_f(gt.x), u.y * up.y * silu_grad_f(gt.y),
+                                                u.z * up.z * silu_grad_f(gt.z), u.w * up.w * silu_grad_f(gt.w)));
+    st4_dt(g.C, g.c_dtype, cc + 64, vec, make_float4(u.x * silu_f(gt.x), u.y * silu_f(gt.y), u.z * silu_f(gt.z), u.w * silu_f(gt.w)));
+    return;
+  }
+  if (g.epi == EPI_MUL || g.epi == EPI_RESID) {
+    const float4 f = ld4_dt(g.aux, g.aux_dtype, (int64_t)m * g.ldaux + n, vec);
+    u = g.epi == EPI_MUL ? make_float4(u.x * f.x, u.y * f.y, u.z * f.z, u.w * f.w)
+                         : make_float4(u.x + f.x, u.y + f.y, u.z + f.z, u.w + f.w);
+  }
+  st4_dt(g.C, g.c_dtype, c, vec, u);
+}
+
+// The fp32 models' GEMMs have a few hundred rows at most (128 to 512 tokens), so time goes to the chain
+// over K on the few SMs that have a tile: the tile is small (32 x 32) and the CTA's 8 warps split K.  A
+// lane holds 8 x 4 sums; each warp copies its own operands through a ring of three 8-deep chunks
+// (cp.async; the accumulation never waits for a whole load) and the warps' tiles are summed in warp
+// order.  Packed FMAs: two k at a time with B [N, K] (both operands come as pairs), two columns with
+// B [K, N].  Measured (64 x 64 tiles, one chain over K, scalar loads before): 128 x 128, K = 128 to 512:
+// 32 -> 6.8 us; 385 x 192, K = 192 to 768: 46 -> 8.8; 385 x 768, K = 192: 22.6 -> 10.4.
+template <typename TI, bool KN>
+__global__ void __launch_bounds__(NT, 2) gemm_simt_kernel(GemmArgs g, int ks, bool va, bool vb, bool vc) {
+  constexpr int LDA = sizeof(TI) == 4 ? KC + 4 : KC;  // elements
+  constexpr int LDB = KN ? BT : LDA;
+  constexpr int ASZ = BT * LDA, STAGE = ASZ + (KN ? KC : BT) * LDB;
+  extern __shared__ __align__(16) uint8_t smb[];
+  pdl_wait();
+  pdl_trigger();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, lr = lane >> 3, lc = lane & 7;
+  const int m0 = blockIdx.y * BT, n0 = blockIdx.x * BT;
   const TI* A = reinterpret_cast<const TI*>(g.A);
   const TI* B = reinterpret_cast<const TI*>(g.B);
-  float acc[4][4];
+  const int k0 = warp * ks, k1 = min(g.K, k0 + ks), n = k0 < k1 ? (k1 - k0 + KC - 1) / KC : 0;
+  TI* ring = reinterpret_cast<TI*>(smb) + warp * NS * STAGE;
+  auto issue = [&](int i) {
+    if (i < n) {
+      TI* st = ring + (i % NS) * STAGE;
+      const int k = k0 + i * KC;
+      copy_block(st, LDA, A + (size_t)m0 * g.lda + k, (size_t)g.lda, BT, KC, g.M - m0, k1 - k, va, lane);
+      if (KN) copy_block(st + ASZ, LDB, B + (size_t)k * g.ldb + n0, (size_t)g.ldb, KC, BT, k1 - k, g.N - n0, vb, lane);
+      else copy_block(st + ASZ, LDB, B + (size_t)n0 * g.ldb + k, (size_t)g.ldb, BT, KC, g.N - n0, k1 - k, vb, lane);
+    }
+    cp_commit();
+  };
+  // KN: acc[i][j] = columns 4 lc + 2 j, + 1 (j < 2); else the even and odd k of column lc + 8 j
+  float2 acc[8][4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < 8; ++i) acc[i][0] = acc[i][1] = acc[i][2] = acc[i][3] = make_float2(0.f, 0.f);
+  for (int i = 0; i < NS - 1; ++i) issue(i);
+#pragma unroll 1
+  for (int i = 0; i < n; ++i) {
+    cp_wait<NS - 2>();
+    __syncwarp();
+    issue(i + NS - 1);  // (its stage was read before this __syncwarp)
+    const TI* as = ring + (i % NS) * STAGE;
+    const TI* bs = as + ASZ;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-
-  for (int k0 = 0; k0 < g.K; k0 += BK) {
-    // 64 x 16 tiles: 1024 elements, 4 per thread; k fastest for coalescing
+    for (int kq = 0; kq < KC; kq += 4) {
+      float4 b[4];
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      int e = tid + r * NT;
-      int row = e >> 4, kk = e & 15;
-      int gm = m0 + row, gk = k0 + kk;
-      As[kk][row] = (gm < g.M && gk < g.K) ? to_f(A[(int64_t)gm * g.lda + gk]) : 0.f;
-      if (g.b_kn) {  // B stored [K, N]: n fastest for coalescing
-        int n = e & 63, k = e >> 6, gn = n0 + n, gk2 = k0 + k;
-        Bs[k][n] = (gn < g.N && gk2 < g.K) ? to_f(B[(int64_t)gk2 * g.ldb + gn]) : 0.f;
-      } else {
-        int gn = n0 + row;
-        Bs[kk][row] = (gn < g.N && gk < g.K) ? to_f(B[(int64_t)gn * g.ldb + gk]) : 0.f;
+      for (int j = 0; j < 4; ++j) b[j] = KN ? ld4s(bs + (kq + j) * LDB + 4 * lc) : ld4s(bs + (lc + 8 * j) * LDB + kq);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const float4 x = ld4s(as + (lr + 4 * q) * LDA + kq);
+        if (KN) {
+          const float xv[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk) {
+            acc[q][0] = __ffma2_rn(f2(xv[kk]), make_float2(b[kk].x, b[kk].y), acc[q][0]);
+            acc[q][1] = __ffma2_rn(f2(xv[kk]), make_float2(b[kk].z, b[kk].w), acc[q][1]);
+          }
+        } else {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            acc[q][j] = __ffma2_rn(make_float2(x.x, x.y), make_float2(b[j].x, b[j].y), acc[q][j]);
+            acc[q][j] = __ffma2_rn(make_float2(x.z, x.w), make_float2(b[j].z, b[j].w), acc[q][j]);
+          }
+        }
       }
     }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      float a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-    }
-    __syncthreads();
   }
+  cp_wait<0>();
+  __syncthreads();  // every ring is read: the warps' tiles take their place
+  float* part = reinterpret_cast<float*>(smb);
+  if (n > 0) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    int m = m0 + ty + 16 * i;
-    if (m >= g.M) continue;
+    for (int q = 0; q < 8; ++q) {
+      float* row = part + (warp * BT + lr + 4 * q) * LDP;
+      if (KN) {
+        *reinterpret_cast<float4*>(row + 4 * lc) = make_float4(acc[q][0].x, acc[q][0].y, acc[q][1].x, acc[q][1].y);
+      } else {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      int n = n0 + tx + 16 * j;
-      if (n < g.N) epilogue(g, m, n, acc[i][j]);
+        for (int j = 0; j < 4; ++j) row[lc + 8 * j] = acc[q][j].x + acc[q][j].y;
+      }
     }
   }
+  __syncthreads();
+  const int nk = (g.K + ks - 1) / ks, r = threadIdx.x >> 3, c = (threadIdx.x & 7) * 4;
+  const int m = m0 + r, col = n0 + c;
+  if (m >= g.M || col >= g.N) return;
+  float4 s = *reinterpret_cast<const float4*>(part + r * LDP + c);
+  for (int w = 1; w < nk; ++w) {
+    const float4 t = *reinterpret_cast<const float4*>(part + (w * BT + r) * LDP + c);
+    s.x += t.x; s.y += t.y; s.z += t.z; s.w += t.w;
+  }
+  if (col + 3 < g.N) {
+    epilogue4(g, m, col, s, vc);
+  } else {
+    const float v[4] = {s.x, s.y, s.z, s.w};
+    for (int i = 0; i < 4 && col + i < g.N; ++i) epilogue(g, m, col + i, v[i]);
+  }
+}
+
+template <typename TI, bool KN>
+cudaError_t launch_simt(const GemmArgs& g, cudaStream_t st) {
+  constexpr int LDA = sizeof(TI) == 4 ? KC + 4 : KC, E = 16 / (int)sizeof(TI);
+  constexpr size_t ring = (size_t)NW * NS * (BT * LDA + (KN ? KC * BT : BT * LDA)) * sizeof(TI), part = (size_t)NW * BT * LDP * 4;
+  constexpr size_t smem = ring > part ? ring : part;
+  auto k = gemm_simt_kernel<TI, KN>;
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  const int ks = ((g.K + NW - 1) / NW + KC - 1) / KC * KC;
+  auto al = [](const void* p, int ld) { return ((uintptr_t)p & 15) == 0 && ld % 4 == 0; };
+  const bool va = g.K % E == 0 && g.lda % E == 0 && ((uintptr_t)g.A & 15) == 0;
+  const bool vb = (KN ? g.N : g.K) % E == 0 && g.ldb % E == 0 && ((uintptr_t)g.B & 15) == 0;
+  const bool vc = al(g.C, g.ldc) && al(g.C2, g.ldc2) && al(g.aux, g.ldaux);
+  e = launch_pdl(k, dim3((g.N + BT - 1) / BT, (g.M + BT - 1) / BT), dim3(NT), smem, st, g, ks, va, vb, vc);
+  note_launch(1);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 // h[m, j] = silu(gate) * up from the packed [gate|up] matrix
@@ -135,11 +242,8 @@ __global__ void swiglu_kernel(const void* gu, int ld_gu, int gu_dtype, void* h, 
 
 cudaError_t gemm_simt(const GemmArgs& g, cudaStream_t st) {
   if (g.M <= 0 || g.N <= 0) return cudaSuccess;
-  dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM);
-  if (g.in_dtype == DT_BF16) gemm_simt_kernel<bf16><<<grid, NT, 0, st>>>(g);
-  else gemm_simt_kernel<float><<<grid, NT, 0, st>>>(g);
-  note_launch(1);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = g.in_dtype == DT_BF16 ? (g.b_kn ? launch_simt<bf16, true>(g, st) : launch_simt<bf16, false>(g, st))
+                                        : (g.b_kn ? launch_simt<float, true>(g, st) : launch_simt<float, false>(g, st));
   if (e != cudaSuccess || g.epi != EPI_SWIGLU) return e;
   int F = g.N / 2;
   int64_t n = (int64_t)g.M * F;
