@@ -388,11 +388,18 @@ __global__ void __launch_bounds__(HEAD_FWD_THREADS) encoder_head_fwd_kernel(cons
     int lab = labels[b];
     if (lab < 0 || lab >= C) { set_dev_error(err, RA_DEVERR_BOUNDS); lab = 0; }
     red[b] = lse - lg[b * C + lab];
+    // softmax - onehot without the cancellation of p - 1: the label's entry is minus the others' sum
+    // (the bias gradient adds these up over the batch and nearly cancels)
+    float others = 0.f;
     for (int c = 0; c < C; ++c) {
-      if (logits_out) logits_out[b * C + c] = lg[b * C + c];
-      float p = expf(lg[b * C + c] - lse);
-      dlogits[b * C + c] = (p - (c == lab ? 1.f : 0.f)) / B;
+      const float l = lg[b * C + c], e = expf(l - mx);
+      if (logits_out) logits_out[b * C + c] = l;
+      if (c != lab) {
+        others += e;
+        dlogits[b * C + c] = e / se / B;
+      }
     }
+    dlogits[b * C + lab] = -(others / se / B);
   }
   __syncthreads();
   if (threadIdx.x == 0) {
