@@ -10,7 +10,7 @@
 //   warp 0      TMA producer: 128 x 64 A tiles and BN x 64 B tiles (BN = 128, 192 or 256;
 //               128-byte swizzle) into a STAGES-deep shared-memory ring, completion tracked
 //               by mbarrier tx counts;
-//   warp 1      allocates 2*BN TMEM columns (two accumulators); one thread issues
+//   warp 1      allocates 2*BN TMEM columns (two accumulators); one lane issues
 //               tcgen05.mma (M = 128, N = BN, K = 16) and tcgen05.commit to free each stage
 //               and to publish each finished accumulator;
 //   warps 2..9  epilogue: two warps per TMEM lane quadrant (warp w may only read lanes
@@ -27,6 +27,7 @@
 #include <algorithm>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 #include <unordered_map>
 
 #include "common.cuh"
@@ -469,7 +470,7 @@ __global__ void __launch_bounds__(EpiTraits<EPI>::THREADS, 1)
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   const uint32_t smem_base = smem_u32(smem);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -512,11 +513,9 @@ __global__ void __launch_bounds__(EpiTraits<EPI>::THREADS, 1)
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
-    if (lane == 0) {
-      int stage = 0;
+    if (elect_one()) {
+      int stage = 0, issued = 0;
       uint32_t phase = 0;
-      int pending_phase[STAGES];
-      for (int s = 0; s < STAGES; ++s) pending_phase[s] = -1;
       bool ok = true;
       for (int u = 0; ok && u < sch.count(); ++u) {
         int tile, kb0, kb1, kind;
@@ -539,56 +538,61 @@ __global__ void __launch_bounds__(EpiTraits<EPI>::THREADS, 1)
           } else {
             tma_load_2d(&tmB, sa + Cfg::A_BYTES, &full_bar[stage], kb * BK, n0);
           }
-          pending_phase[stage] = (int)phase;
+          ++issued;
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
       }
       if (!ok) {  // let every copy this thread started land before the CTA goes away
         volatile int no_abort = 0;
-        for (int s = 0; s < STAGES; ++s)
-          if (pending_phase[s] >= 0) mbar_wait(&full_bar[s], (uint32_t)pending_phase[s], &no_abort, nullptr);
+        for (int i = max(0, issued - STAGES); i < issued; ++i)
+          mbar_wait(&full_bar[i % STAGES], (uint32_t)(i / STAGES) & 1u, &no_abort, nullptr);
       }
     }
+    __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      const uint32_t idesc = p.b_kn ? idesc_bf16_bmn(BM, BN) : idesc_bf16(BM, BN);
-      int stage = 0;
-      uint32_t phase = 0;
-      int acc = 0;
-      uint32_t acc_phase = 0;
-      bool ok = true;
-      for (int u = 0; ok && u < sch.count(); ++u) {
-        int tile, kb0, kb1, kind;
-        sch.unit(u, tile, kb0, kb1, kind);
-        if (!mbar_wait(&tempty_bar[acc], acc_phase ^ 1u, &abort_sh, p.err)) break;
-        tc_fence_after();
-        const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
-        for (int kb = kb0; kb < kb1; ++kb) {
-          if (!mbar_wait(&full_bar[stage], phase, &abort_sh, p.err)) { ok = false; break; }
+    if (elect_one()) {
+      const uint64_t ring = sdesc_sw128(smem_base), ring_kn = sdesc_mn_sw128_lbo(smem_base, 8192);
+      auto issue = [&](auto kn) {  // KN: B as stored [K, N]
+        constexpr bool KN = decltype(kn)::value;
+        constexpr uint32_t idesc = KN ? idesc_bf16_bmn(BM, BN) : idesc_bf16(BM, BN);
+        // K-major B: advance 16 elements = 32 bytes inside the swizzle atom; [K, N] B
+        // (MN-major): advance 16 rows = 2048 bytes, atoms along N 8 KB apart
+        constexpr uint64_t bstep = KN ? 128u : 2u;
+        int stage = 0;
+        uint32_t phase = 0;
+        int acc = 0;
+        uint32_t acc_phase = 0;
+        for (int u = 0; u < sch.count(); ++u) {
+          int tile, kb0, kb1, kind;
+          sch.unit(u, tile, kb0, kb1, kind);
+          if (!mbar_wait(&tempty_bar[acc], acc_phase ^ 1u, &abort_sh, p.err)) return;
           tc_fence_after();
-          const uint32_t sa = smem_base + stage * Cfg::STAGE_BYTES;
-          const uint64_t adesc = sdesc_sw128(sa);
-          // K-major B: advance 16 elements = 32 bytes inside the swizzle atom; [K, N] B
-          // (MN-major): advance 16 rows = 2048 bytes, atoms along N 8 KB apart
-          const uint64_t bdesc = p.b_kn ? sdesc_mn_sw128_lbo(sa + Cfg::A_BYTES, 8192) : sdesc_sw128(sa + Cfg::A_BYTES);
-          const uint64_t bstep = p.b_kn ? 128u : 2u;
+          const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
+          for (int kb = kb0; kb < kb1; ++kb) {
+            if (!mbar_wait(&full_bar[stage], phase, &abort_sh, p.err)) return;
+            tc_fence_after();
+            const uint64_t off = (uint64_t)(stage * (Cfg::STAGE_BYTES / 16));
+            const uint64_t adesc = ring + off, bdesc = (KN ? ring_kn : ring) + off + (uint64_t)(Cfg::A_BYTES / 16);
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k)
-            umma_bf16(d_tmem, adesc + (uint64_t)(2 * k), bdesc + bstep * (uint64_t)k, idesc,
-                      (kb != kb0 || k != 0) ? 1u : 0u);
-          umma_commit(&empty_bar[stage]);
-          if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+            for (int k = 0; k < BK / 16; ++k)
+              umma_bf16(d_tmem, adesc + (uint64_t)(2 * k), bdesc + bstep * (uint64_t)k, idesc,
+                        (kb != kb0 || k != 0) ? 1u : 0u);
+            umma_commit(&empty_bar[stage]);
+            if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+          }
+          umma_commit(&tfull_bar[acc]);
+          if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
-        if (!ok) break;
-        umma_commit(&tfull_bar[acc]);
-        if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
-      }
+      };
+      if (p.b_kn) issue(std::true_type());
+      else issue(std::false_type());
       // all MMAs issued by this thread complete before TMEM and shared memory are released
       umma_commit(&drain_bar);
       volatile int no_abort = 0;
       mbar_wait(&drain_bar, 0, &no_abort, nullptr);
     }
+    __syncwarp();
   } else {
     // ------------------------------------------------------------------ epilogue (warps 2..9)
     const int quad = warp & 3;             // TMEM lanes 32*quad .. 32*quad + 31
@@ -643,7 +647,7 @@ __global__ void __launch_bounds__(EpiTraits<EPI>::THREADS, 1)
       if ((EPI == EPI_STORE || EPI == EPI_BIAS_GELU || EPI == EPI_BIAS_GELU_G) && p.bias &&
           half + PARTS * lane < BN / 32 && n0 + 32 * (half + PARTS * lane) < p.N)
         asm volatile("prefetch.global.L1 [%0];" ::"l"(p.bias + n0 + 32 * (half + PARTS * lane)));
-      if (!mbar_wait(&tfull_bar[acc], acc_phase, &abort_sh, p.err)) break;
+      if (!mbar_wait_warp(&tfull_bar[acc], acc_phase, &abort_sh, p.err)) break;
       tc_fence_after();
       const uint32_t tbase = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * BN);
       // finisher: the partials of CTAs src0 .. blockIdx.x - 1 (this warp's rows and columns)
@@ -684,7 +688,7 @@ __global__ void __launch_bounds__(EpiTraits<EPI>::THREADS, 1)
           tmem_ld32_issue(tbase + c0, r);
           const int reg = (aux_i - 1) % nreg;        // region of this chunk's operand
           uint8_t* region = staging + reg * rbytes;
-          if (!mbar_wait(&abar[reg], aux_phase[reg], &abort_sh, p.err)) { ok = false; tmem_wait32(r); break; }
+          if (!mbar_wait_warp(&abar[reg], aux_phase[reg], &abort_sh, p.err)) { ok = false; tmem_wait32(r); break; }
           aux_phase[reg] ^= 1u;
           ++aux_waited;
           float x1[32], x2[32];
@@ -1013,16 +1017,17 @@ cudaError_t gemm_tc(const GemmArgs& g, cudaStream_t st) {
 
   const int sms = device_sm_count();
   const int m_tiles = (g.M + BM - 1) / BM;
-  // tile width: fewest waves of 128 x BN tiles (time ~ waves x BN), weighting the narrower
-  // tiles by their measured cost per column: a 128-wide tile carries more shared-memory
-  // operand traffic per flop, and a 192-wide tile takes about as long as a 256-wide one
-  // (measured: 0.96x the time of a 256-wide tile).  So 192 wins only where it saves a
-  // whole wave at equal count, e.g. N = 768 at 4096 rows: 128 tiles in one wave instead of
-  // 96 tiles of 256 columns on a third fewer SMs.
+  // Tile width: fewest waves of 128 x BN tiles, weighted by each width's measured time per column
+  // and k-block (8192 x 3072 and 4096 x 3072, K = 768 and 1024: 0.22 us at 128 columns, 0.31 at
+  // 192, 0.365 at 256; the issue of the products and copies paces the narrow ones).  192 wins where
+  // it saves a wave or fills it (4096 x 768, K = 3072: 16.8 us against 19.1 at 256 and 22.9 at 128).
+  // Under the GELU epilogues the epilogue sets the pace and 192 costs no more per column than 256
+  // (8192 x 3072, K = 1024: 49.6 us at 192, 54.2 at 256; 4096 x 3072, K = 768: 29.7 and 31.0).
+  const bool gelu = g.epi == EPI_BIAS_GELU || g.epi == EPI_BIAS_GELU_G;
   auto cost = [&](int bn) {
     int tiles = m_tiles * ((g.N + bn - 1) / bn);
     int waves = (tiles + sms - 1) / sms;
-    return (double)waves * bn * (bn == 128 ? 1.15 : bn == 192 ? 1.27 : 1.0);
+    return (double)waves * bn * (bn == 128 ? 1.22 : bn == 192 ? (gelu ? 0.99 : 1.14) : 1.0);
   };
   int BNsel = (g.N <= 128 || cost(128) < cost(256)) ? 128 : 256;
   if (g.N > 128 && g.epi != EPI_SWIGLU && g.epi != EPI_DSWIGLU && cost(192) < cost(BNsel)) BNsel = 192;
