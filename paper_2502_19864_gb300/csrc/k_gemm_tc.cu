@@ -1014,6 +1014,9 @@ cudaError_t gemm_tc(const GemmArgs& g, cudaStream_t st) {
   if (g.epi == EPI_DSWIGLU && g.N % 64) return cudaErrorNotSupported;
   if (!has_c && g.epi != EPI_BIAS_GELU && g.epi != EPI_BIAS_GELU_G && g.epi != EPI_SWIGLU)
     return cudaErrorNotSupported;
+  // few tiles: K split over clusters
+  const cudaError_t few = gemm_splitk(g, st);
+  if (few != cudaErrorNotSupported) return few;
 
   const int sms = device_sm_count();
   const int m_tiles = (g.M + BM - 1) / BM;

@@ -83,6 +83,8 @@ int gemm_sk_flags_per_slot();
 cudaError_t gemm(const GemmArgs& a, cudaStream_t st);
 // tcgen05 path; returns cudaErrorNotSupported if the shape/dtype is not handled.
 cudaError_t gemm_tc(const GemmArgs& a, cudaStream_t st);
+// the form of gemm_tc for few output tiles (it decides); cudaErrorNotSupported otherwise
+cudaError_t gemm_splitk(const GemmArgs& a, cudaStream_t st);
 cudaError_t gemm_simt(const GemmArgs& a, cudaStream_t st);
 // Bounded-wait self-test (failure detection): a wait that nothing satisfies runs out after
 // limit_ns and sets RA_DEVERR_TIMEOUT in *err.
