@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(NTHR, DH == 64 ? 2 : 1) attn_bwd_tc_kernel(Att
     if (threadIdx.x == 0) set_dev_error(a.err, RA_DEVERR_BOUNDS);
     return;
   }
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const int quad = warp & 3, half = warp >> 2;  // TMEM lane quadrant; 64-column half of a block
   const int bh = blockIdx.x, b = bh / a.n_heads, hh = bh % a.n_heads;
   const bool keys = blockIdx.y == 0;
@@ -300,7 +300,7 @@ __global__ void __launch_bounds__(NTHR, DH == 64 ? 2 : 1) attn_bwd_tc_kernel(Att
       load_stats(i * BR);
       copies_done();
       publish();
-      if (tid == 0) {  // S^T = k_j q_i^T
+      if (warp == 0 && elect_one()) {  // S^T = k_j q_i^T
         mma_qk<DH>(tmem + Pl::C_S, sb + Pl::T0, sb + Pl::T2, ID128);
         umma_commit(&bar);
       }
@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(NTHR, DH == 64 ? 2 : 1) attn_bwd_tc_kernel(Att
       if (!ok) break;
       softmax_to_x(j * BR, i * BR);  // P^T
       publish();
-      if (tid == 0) {  // dV_j += P^T dO_i; dP^T = v_j dO_i^T
+      if (warp == 0 && elect_one()) {  // dV_j += P^T dO_i; dP^T = v_j dO_i^T
         mma_xb<DH>(tmem + Pl::C_A, sb + Pl::X, sb + Pl::T3, i > i_first);
         mma_qk<DH>(tmem + Pl::C_S, sb + Pl::T1, sb + Pl::T3, ID128);
         umma_commit(&bar);
@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(NTHR, DH == 64 ? 2 : 1) attn_bwd_tc_kernel(Att
       if (!ok) break;
       ds_in_x();  // dS^T over P^T (dV has read it)
       publish();
-      if (tid == 0) {  // dK_j += dS^T q_i
+      if (warp == 0 && elect_one()) {  // dK_j += dS^T q_i
         mma_xb<DH>(tmem + Pl::C_B, sb + Pl::X, sb + Pl::T2, i > i_first);
         umma_commit(&bar);
       }
@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(NTHR, DH == 64 ? 2 : 1) attn_bwd_tc_kernel(Att
       load_block<DH>(sb + Pl::T3, qkv + 2 * H, ld, j * BR, S); // v_j
       copies_done();
       publish();
-      if (tid == 0) {  // S = q_i k_j^T
+      if (warp == 0 && elect_one()) {  // S = q_i k_j^T
         mma_qk<DH>(tmem + Pl::C_S, sb + Pl::T0, sb + Pl::T2, ID128);
         umma_commit(&bar);
       }
@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(NTHR, DH == 64 ? 2 : 1) attn_bwd_tc_kernel(Att
       if (!ok) break;
       softmax_to_x(i * BR, j * BR);  // P (rows = queries)
       publish();  // S read before dP overwrites it
-      if (tid == 0) {  // dP = dO_i v_j^T
+      if (warp == 0 && elect_one()) {  // dP = dO_i v_j^T
         mma_qk<DH>(tmem + Pl::C_S, sb + Pl::T1, sb + Pl::T3, ID128);
         umma_commit(&bar);
       }
@@ -362,7 +362,7 @@ __global__ void __launch_bounds__(NTHR, DH == 64 ? 2 : 1) attn_bwd_tc_kernel(Att
       if (!ok) break;
       ds_in_x();  // dS over P
       publish();
-      if (tid == 0) {  // dQ_i += dS k_j
+      if (warp == 0 && elect_one()) {  // dQ_i += dS k_j
         mma_xb<DH>(tmem + Pl::C_A, sb + Pl::X, sb + Pl::T2, j > 0);
         umma_commit(&bar);
       }
@@ -442,7 +442,7 @@ __global__ void __launch_bounds__(NTHR, 2) attn_fwd_blocks_tc_kernel(AttnArgs a)
     if (threadIdx.x == 0) set_dev_error(a.err, RA_DEVERR_BOUNDS);
     return;
   }
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const int quad = warp & 3, half = warp >> 2;
   const int S = a.S, NB = (S + BR - 1) / BR;
   const int i = NB - 1 - (int)blockIdx.x, bh = blockIdx.y, b = bh / a.n_heads, hh = bh % a.n_heads;
@@ -507,7 +507,7 @@ __global__ void __launch_bounds__(NTHR, 2) attn_fwd_blocks_tc_kernel(AttnArgs a)
     load_block<DH>(sb + Pl::K, qkv + H, ld, j * BR, S);
     copies_done();
     publish();
-    if (tid == 0) {
+    if (warp == 0 && elect_one()) {
       mma_qk<DH>(tmem + Pl::C_S, sb + Pl::Q, sb + Pl::K, ID128);
       umma_commit(&bar);
     }
@@ -559,7 +559,7 @@ __global__ void __launch_bounds__(NTHR, 2) attn_fwd_blocks_tc_kernel(AttnArgs a)
     asm volatile("cp.async.commit_group;" ::: "memory");
     asm volatile("cp.async.wait_group 1;" ::: "memory");      // k_j
     publish();
-    if (tid == 0) {
+    if (warp == 0 && elect_one()) {
       mma_qk<DH>(tmem + Pl::C_S, sb + Pl::Q, sb + Pl::K, ID128);
       umma_commit(&bar);
     }
@@ -590,7 +590,7 @@ __global__ void __launch_bounds__(NTHR, 2) attn_fwd_blocks_tc_kernel(AttnArgs a)
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");  // v_j
     publish();
-    if (tid == 0) {
+    if (warp == 0 && elect_one()) {
       mma_xb<DH>(tmem + Pl::C_O, sb + Pl::X, sb + Pl::V, j > 0);
       umma_commit(&bar);
     }

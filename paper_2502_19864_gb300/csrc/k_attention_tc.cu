@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(256) attn_fwd_tc_kernel(const __grid_constant_
     if (threadIdx.x == 0) set_dev_error(a.err, RA_DEVERR_BOUNDS);
     return;
   }
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const int quad = warp & 3, half = warp >> 2;  // TMEM lane quadrant, column half
   const int bh = blockIdx.y, b = bh / a.n_heads, hh = bh % a.n_heads;
   const int H = a.n_heads * DH, S = a.S;
@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(256) attn_fwd_tc_kernel(const __grid_constant_
   pdl_trigger();
 
   // q, k and v: one box each from the [B S, 3 H] qkv matrix (x = the head's columns)
-  if (tid == 0) {
+  if (warp == 0 && elect_one()) {
     mbar_expect_tx(&load_bar, (uint32_t)(QT + 2 * NK) * 128);
     tma_load_2d_at(&tmQ, sbase + Pl::Q_OFF, &load_bar, hh * DH, b * S + q0);
     tma_load_2d_at(&tmKV, sbase + Pl::K_OFF, &load_bar, H + hh * DH, b * S);
@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(256) attn_fwd_tc_kernel(const __grid_constant_
   tc_fence_after();
 
   // S = q k^T
-  if (tid == 0 && ok) {
+  if (warp == 0 && elect_one() && ok) {
     constexpr uint32_t idesc = idesc_bf16(QT, NK);
     const uint64_t ad = sdesc_sw128(sbase + Pl::Q_OFF), bd = sdesc_sw128(sbase + Pl::K_OFF);
 #pragma unroll
@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(256) attn_fwd_tc_kernel(const __grid_constant_
   sum = red[0][row] + red[1][row];
 
   // O = p v into TMEM columns [0, 64) (S is no longer read)
-  if (tid == 0 && ok) {
+  if (warp == 0 && elect_one() && ok) {
     constexpr uint32_t idesc = idesc_bf16_bmn(QT, DH);
 #pragma unroll
     for (int kk = 0; kk < NK / 16; ++kk) {
