@@ -6,7 +6,7 @@
 // backward (fused GELU' / SwiGLU' / residual epilogues) -- the dense contractions of the
 // step.
 //
-// Structure (one persistent CTA per SM, 320 threads):
+// Structure (one persistent CTA per SM, 320 threads; large products in pairs of CTAs, see CG below):
 //   warp 0      TMA producer: 128 x 64 A tiles and BN x 64 B tiles (BN = 128, 192 or 256;
 //               128-byte swizzle) into a STAGES-deep shared-memory ring, completion tracked
 //               by mbarrier tx counts;
@@ -62,13 +62,15 @@ struct EpiTraits {
 // epilogues TMA-load their operand chunk into that area: bf16 factor operands use two 2 KB
 // regions (the next chunk loads while this one computes); 4 KB operands (fp32 residual,
 // packed gate|up) use one region, whose first chunk per tile loads during the main loop.
-template <int BN, bool AUX, int EW = 8>
+template <int BN, bool AUX, int EW = 8, int CG = 1>
 struct TileCfg {
   // the operand ring gives up a stage to the staging of the extra epilogue warps (a
-  // 192-wide ring keeps 4 stages either way: 40 KB stages)
-  static constexpr int STAGES = BN == 256 ? (EW > 8 ? 3 : 4) : BN == 192 ? 4 : (EW > 8 ? 5 : 6);
+  // 192-wide ring keeps 4 stages either way: 40 KB stages); a CTA of a pair holds half of B
+  static constexpr int STAGES = CG == 2 ? (EW > 8 ? 5 : 6)
+                              : BN == 256 ? (EW > 8 ? 3 : 4) : BN == 192 ? 4 : (EW > 8 ? 5 : 6);
   static constexpr int A_BYTES = BM * BK * 2;
-  static constexpr int B_BYTES = BN * BK * 2;
+  static constexpr int BNC = BN / CG;  // columns of B in this CTA
+  static constexpr int B_BYTES = BNC * BK * 2;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
   // two accumulators of BN columns; the allocation is a power of two
   static constexpr int TMEM_COLS = 2 * BN <= 256 ? 256 : 512;
@@ -177,6 +179,23 @@ __device__ __forceinline__ void tma_load_3d(const CUtensorMap* tm, uint32_t dst,
       "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
       " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
       "l"(reinterpret_cast<uint64_t>(tm)), "r"(c0), "r"(c1), "r"(c2), "r"(smem_u32(bar))
+      : "memory");
+}
+// the same into this CTA of a pair, completing on the barrier at a shared::cluster address (the
+// leader's)
+__device__ __forceinline__ void tma_load_2d_pair(const CUtensorMap* tm, uint32_t dst, uint32_t bar, int c0, int c1) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(tm)), "r"(c0), "r"(c1), "r"(bar)
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_3d_pair(const CUtensorMap* tm, uint32_t dst, uint32_t bar, int c0, int c1,
+                                                 int c2) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(tm)), "r"(c0), "r"(c1), "r"(c2), "r"(bar)
       : "memory");
 }
 __device__ __forceinline__ void tma_store_2d(const CUtensorMap* tm, uint32_t src, int c0, int c1) {
@@ -452,13 +471,16 @@ __device__ __forceinline__ void tile_coords(int tile, int m_tiles, int n_tiles, 
 }
 
 // ---- the kernel -------------------------------------------------------------------------------
-template <int BN, int EPI>
+// CG = 2: a cluster of two CTAs works on 2 x 128 rows as one product (tcgen05 cta_group::2): each
+// CTA loads its own 128 rows of A and half of B, the even CTA issues the products for both, and
+// each drains its own 128 rows.  All tiles, units and indexes below are then those of the pair.
+template <int BN, int EPI, int CG>
 __global__ void __launch_bounds__(EpiTraits<EPI>::THREADS, 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                    const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmC2,
                    const __grid_constant__ CUtensorMap tmX, const TcParams p) {
   constexpr int EW = EpiTraits<EPI>::WARPS;
-  using Cfg = TileCfg<BN, EpiTraits<EPI>::AUX, EW>;
+  using Cfg = TileCfg<BN, EpiTraits<EPI>::AUX, EW, CG>;
   constexpr int STAGES = Cfg::STAGES;
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t full_bar[STAGES], empty_bar[STAGES];
@@ -471,6 +493,8 @@ __global__ void __launch_bounds__(EpiTraits<EPI>::THREADS, 1)
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   const uint32_t smem_base = smem_u32(smem);
   const int warp = warp_index(), lane = threadIdx.x & 31;
+  const int rank = CG == 2 ? (int)cluster_rank() : 0;
+  const int cta = (int)blockIdx.x / CG;  // (of the pair, where CTAs work in pairs)
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -479,7 +503,7 @@ __global__ void __launch_bounds__(EpiTraits<EPI>::THREADS, 1)
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(&tfull_bar[a], 1);
-      mbar_init(&tempty_bar[a], EW);
+      mbar_init(&tempty_bar[a], EW * CG);
     }
     mbar_init(&drain_bar, 1);
     for (int w = 0; w < EW; ++w) {
@@ -494,12 +518,25 @@ __global__ void __launch_bounds__(EpiTraits<EPI>::THREADS, 1)
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
   }
+  if (CG == 2) {  // the barriers of both CTAs are there before either signals the other's
+    __syncthreads();
+    cluster_arrive();
+    cluster_wait();
+  }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                     smem_u32(&tmem_base_sh)),
-                 "r"((uint32_t)Cfg::TMEM_COLS)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if (CG == 2) {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                       smem_u32(&tmem_base_sh)),
+                   "r"((uint32_t)Cfg::TMEM_COLS)
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                       smem_u32(&tmem_base_sh)),
+                   "r"((uint32_t)Cfg::TMEM_COLS)
+                   : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
   }
   tc_fence_before();
   __syncthreads();
@@ -509,7 +546,7 @@ __global__ void __launch_bounds__(EpiTraits<EPI>::THREADS, 1)
   pdl_wait();
   pdl_trigger();
   Sched sch;
-  sch.init(p, blockIdx.x, gridDim.x);
+  sch.init(p, cta, (int)gridDim.x / CG);
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
@@ -522,40 +559,60 @@ __global__ void __launch_bounds__(EpiTraits<EPI>::THREADS, 1)
         sch.unit(u, tile, kb0, kb1, kind);
         int mt, nt;
         tile_coords(tile, p.m_tiles, p.n_tiles_n, mt, nt);
-        const int m0 = mt * BM, n0 = nt * BN;
+        const int m0 = (mt * CG + rank) * BM, n0 = nt * BN + rank * Cfg::BNC;
         for (int kb = kb0; kb < kb1; ++kb) {
           if (!mbar_wait(&empty_bar[stage], phase ^ 1u, &abort_sh, p.err)) { ok = false; break; }
-          mbar_expect_tx(&full_bar[stage], Cfg::STAGE_BYTES);
+          if (rank == 0) mbar_expect_tx(&full_bar[stage], CG * Cfg::STAGE_BYTES);
           const uint32_t sa = smem_base + stage * Cfg::STAGE_BYTES;
-          tma_load_2d(&tmA, sa, &full_bar[stage], kb * BK, m0);
-          if (p.b_kn == 2) {
-            tma_load_3d(&tmB, sa + Cfg::A_BYTES, &full_bar[stage], 0, kb * BK, n0 / 64);
-          } else if (p.b_kn) {
-            // rows kb*BK.. of B [K, N]: one 64-column swizzle atom (8 KB) per 64 columns
+          if (CG == 2) {
+            const uint32_t full = peer_addr(smem_u32(&full_bar[stage]), 0);
+            tma_load_2d_pair(&tmA, sa, full, kb * BK, m0);
+            if (p.b_kn == 2) {
+              tma_load_3d_pair(&tmB, sa + Cfg::A_BYTES, full, 0, kb * BK, n0 / 64);
+            } else if (p.b_kn) {
 #pragma unroll
-            for (int a = 0; a < BN / 64; ++a)
-              tma_load_2d(&tmB, sa + Cfg::A_BYTES + a * 8192, &full_bar[stage], n0 + 64 * a, kb * BK);
+              for (int a = 0; a < Cfg::BNC / 64; ++a)
+                tma_load_2d_pair(&tmB, sa + Cfg::A_BYTES + a * 8192, full, n0 + 64 * a, kb * BK);
+            } else {
+              tma_load_2d_pair(&tmB, sa + Cfg::A_BYTES, full, kb * BK, n0);
+            }
           } else {
-            tma_load_2d(&tmB, sa + Cfg::A_BYTES, &full_bar[stage], kb * BK, n0);
+            tma_load_2d(&tmA, sa, &full_bar[stage], kb * BK, m0);
+            if (p.b_kn == 2) {
+              tma_load_3d(&tmB, sa + Cfg::A_BYTES, &full_bar[stage], 0, kb * BK, n0 / 64);
+            } else if (p.b_kn) {
+              // rows kb*BK.. of B [K, N]: one 64-column swizzle atom (8 KB) per 64 columns
+#pragma unroll
+              for (int a = 0; a < Cfg::BNC / 64; ++a)
+                tma_load_2d(&tmB, sa + Cfg::A_BYTES + a * 8192, &full_bar[stage], n0 + 64 * a, kb * BK);
+            } else {
+              tma_load_2d(&tmB, sa + Cfg::A_BYTES, &full_bar[stage], kb * BK, n0);
+            }
           }
           ++issued;
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
       }
-      if (!ok) {  // let every copy this thread started land before the CTA goes away
+      // let every copy this thread started land before the CTA goes away (of a pair, the even
+      // CTA's barriers count both CTAs' copies, and the odd one leaves after it)
+      if (!ok && rank == 0) {
         volatile int no_abort = 0;
         for (int i = max(0, issued - STAGES); i < issued; ++i)
           mbar_wait(&full_bar[i % STAGES], (uint32_t)(i / STAGES) & 1u, &no_abort, nullptr);
       }
+      // a pair's last signals to this CTA's barriers arrive before it goes away
+      if (CG == 2 && ok)
+        for (int i = max(0, issued - STAGES); i < issued; ++i)
+          mbar_wait(&empty_bar[i % STAGES], (uint32_t)(i / STAGES) & 1u, &abort_sh, p.err);
     }
     __syncwarp();
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    if (elect_one()) {
+    if (rank == 0 && elect_one()) {
       const uint64_t ring = sdesc_sw128(smem_base), ring_kn = sdesc_mn_sw128_lbo(smem_base, 8192);
       auto issue = [&](auto kn) {  // KN: B as stored [K, N]
         constexpr bool KN = decltype(kn)::value;
-        constexpr uint32_t idesc = KN ? idesc_bf16_bmn(BM, BN) : idesc_bf16(BM, BN);
+        constexpr uint32_t idesc = KN ? idesc_bf16_bmn(CG * BM, BN) : idesc_bf16(CG * BM, BN);
         // K-major B: advance 16 elements = 32 bytes inside the swizzle atom; [K, N] B
         // (MN-major): advance 16 rows = 2048 bytes, atoms along N 8 KB apart
         constexpr uint64_t bstep = KN ? 128u : 2u;
@@ -575,20 +632,26 @@ __global__ void __launch_bounds__(EpiTraits<EPI>::THREADS, 1)
             const uint64_t off = (uint64_t)(stage * (Cfg::STAGE_BYTES / 16));
             const uint64_t adesc = ring + off, bdesc = (KN ? ring_kn : ring) + off + (uint64_t)(Cfg::A_BYTES / 16);
 #pragma unroll
-            for (int k = 0; k < BK / 16; ++k)
-              umma_bf16(d_tmem, adesc + (uint64_t)(2 * k), bdesc + bstep * (uint64_t)k, idesc,
-                        (kb != kb0 || k != 0) ? 1u : 0u);
-            umma_commit(&empty_bar[stage]);
+            for (int k = 0; k < BK / 16; ++k) {
+              const uint64_t ak = adesc + (uint64_t)(2 * k), bk = bdesc + bstep * (uint64_t)k;
+              const uint32_t accumulate = (kb != kb0 || k != 0) ? 1u : 0u;
+              if (CG == 2) umma_bf16_pair(d_tmem, ak, bk, idesc, accumulate);
+              else umma_bf16(d_tmem, ak, bk, idesc, accumulate);
+            }
+            if (CG == 2) umma_commit_pair(&empty_bar[stage]);
+            else umma_commit(&empty_bar[stage]);
             if (++stage == STAGES) { stage = 0; phase ^= 1u; }
           }
-          umma_commit(&tfull_bar[acc]);
+          if (CG == 2) umma_commit_pair(&tfull_bar[acc]);
+          else umma_commit(&tfull_bar[acc]);
           if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         }
       };
       if (p.b_kn) issue(std::true_type());
       else issue(std::false_type());
       // all MMAs issued by this thread complete before TMEM and shared memory are released
-      umma_commit(&drain_bar);
+      if (CG == 2) umma_commit_pair_own(&drain_bar);
+      else umma_commit(&drain_bar);
       volatile int no_abort = 0;
       mbar_wait(&drain_bar, 0, &no_abort, nullptr);
     }
@@ -630,12 +693,23 @@ __global__ void __launch_bounds__(EpiTraits<EPI>::THREADS, 1)
     };
     bool ok = true;
     const int ew = warp - 2;
+    // hands an accumulator back to the issuing warp (of a pair, the even CTA's)
+    auto release = [&](int acc_) {
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) {
+        if (CG == 2) mbar_arrive_cluster(peer_addr(smem_u32(&tempty_bar[acc_]), 0));
+        else mbar_arrive(&tempty_bar[acc_]);
+      }
+    };
+    // stream-K slot and flag index of a lower-indexed worker for this CTA's rows
+    auto slot_of = [&](int worker) { return worker * CG + rank; };
     for (int u = 0; ok && u < sch.count(); ++u) {
       int tile, kb0, kb1, kind;
       sch.unit(u, tile, kb0, kb1, kind);
       int mt, nt;
       tile_coords(tile, p.m_tiles, p.n_tiles_n, mt, nt);
-      const int m0 = mt * BM, n0 = nt * BN;
+      const int m0 = (mt * CG + rank) * BM, n0 = nt * BN;
       const int row0 = m0 + quad * 32;
       const int cbeg = half * (BN / 2), cend = cbeg + BN / 2;
       // the first operand chunk is fetched while the main loop of this tile still runs
@@ -650,14 +724,14 @@ __global__ void __launch_bounds__(EpiTraits<EPI>::THREADS, 1)
       if (!mbar_wait_warp(&tfull_bar[acc], acc_phase, &abort_sh, p.err)) break;
       tc_fence_after();
       const uint32_t tbase = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * BN);
-      // finisher: the partials of CTAs src0 .. blockIdx.x - 1 (this warp's rows and columns)
+      // finisher: the partials of CTAs src0 .. cta - 1 (this warp's rows and columns)
       // must be published before they are added
       const int src0 = (EpiTraits<EPI>::SK && kind == 2) ? Sched::first_source(p, tile - p.dp_tiles) : 0;
       if (EpiTraits<EPI>::SK && kind == 2) {
         bool got = true;
         if (lane == 0)
-          for (int cc = src0; got && cc < (int)blockIdx.x; ++cc)
-            got = sk_wait(p.sk_flags + cc * SK_MAX_WARPS + ew, &abort_sh, p.err);
+          for (int cc = src0; got && cc < cta; ++cc)
+            got = sk_wait(p.sk_flags + slot_of(cc) * SK_MAX_WARPS + ew, &abort_sh, p.err);
         if (!__shfl_sync(0xffffffffu, got ? 1 : 0, 0)) break;
       }
       if (EPI == EPI_SWIGLU) {
@@ -737,11 +811,6 @@ __global__ void __launch_bounds__(EpiTraits<EPI>::THREADS, 1)
         const int nch = (BN / 32 - half + PARTS - 1) / PARTS;
         uint32_t ra[32], rb[32];
         auto col = [&](int i) { return 32 * (half + PARTS * i); };
-        auto release = [&]() {
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&tempty_bar[acc]);
-        };
         auto chunk = [&](int c0, uint32_t* r) {
           if (EpiTraits<EPI>::SK && kind == 1) {  // partial: the fp32 accumulator goes to this CTA's slot
             sk_put(p.sk_ws + (size_t)blockIdx.x * SK_SLOT_FLOATS, c0 / 32, quad * 32 + lane,
@@ -752,8 +821,8 @@ __global__ void __launch_bounds__(EpiTraits<EPI>::THREADS, 1)
           // are clipped by the tensor store
           if (n0 + c0 < p.N && row0 < p.M) {
             if (EpiTraits<EPI>::SK && kind == 2)
-              for (int cc = src0; cc < (int)blockIdx.x; ++cc)
-                sk_add(p.sk_ws + (size_t)cc * SK_SLOT_FLOATS, c0 / 32, quad * 32 + lane,
+              for (int cc = src0; cc < cta; ++cc)
+                sk_add(p.sk_ws + (size_t)slot_of(cc) * SK_SLOT_FLOATS, c0 / 32, quad * 32 + lane,
                        reinterpret_cast<float*>(r));
             EpiIn<EPI> in;
             // (N is a multiple of 8: a group of 8 that starts below N ends below it)
@@ -778,12 +847,12 @@ __global__ void __launch_bounds__(EpiTraits<EPI>::THREADS, 1)
         for (int i = 0; i < nch; i += 2) {
           tmem_wait32(ra);
           if (i + 1 < nch) tmem_ld32_issue(tbase + col(i + 1), rb);
-          else release();
+          else release(acc);
           chunk(col(i), ra);
           if (i + 1 < nch) {
             tmem_wait32(rb);
             if (i + 2 < nch) tmem_ld32_issue(tbase + col(i + 2), ra);
-            else release();
+            else release(acc);
             chunk(col(i + 1), rb);
           }
         }
@@ -800,14 +869,12 @@ __global__ void __launch_bounds__(EpiTraits<EPI>::THREADS, 1)
           // them only after this grid has completed)
           __syncwarp();
           if (lane == 0)
-            for (int cc = src0; cc < (int)blockIdx.x; ++cc) p.sk_flags[cc * SK_MAX_WARPS + ew] = 0u;
+            for (int cc = src0; cc < cta; ++cc) p.sk_flags[slot_of(cc) * SK_MAX_WARPS + ew] = 0u;
         }
         if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
         continue;
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&tempty_bar[acc]);
+      release(acc);
       if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
     }
     // an operand load issued but not consumed (only after an abort) lands before exit
@@ -822,7 +889,16 @@ __global__ void __launch_bounds__(EpiTraits<EPI>::THREADS, 1)
 
   tc_fence_before();
   __syncthreads();
-  if (warp == 1) {
+  if (CG == 2) {  // neither CTA leaves while the other may read its operands or signal its barriers
+    cluster_arrive();
+    cluster_wait();
+    if (warp == 1) {
+      tc_fence_after();
+      asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base),
+                   "r"((uint32_t)Cfg::TMEM_COLS)
+                   : "memory");
+    }
+  } else if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base),
                  "r"((uint32_t)Cfg::TMEM_COLS)
@@ -927,41 +1003,53 @@ bool make_map(CUtensorMap* out, const void* ptr, int64_t rows, int64_t cols, int
   return true;
 }
 
-template <int BN, int EPI>
+template <int BN, int EPI, int CG>
 cudaError_t launch(const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& c,
                    const CUtensorMap& c2, const CUtensorMap& x, const TcParams& p, int grid,
                    cudaStream_t st) {
+  using E = EpiTraits<EPI>;
+  constexpr int SMEM = TileCfg<BN, E::AUX, E::WARPS, CG>::SMEM;
+  auto k = gemm_tc_kernel<BN, EPI, CG>;
   static bool attr_set = false;
   if (!attr_set) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<BN, EPI>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         TileCfg<BN, EpiTraits<EPI>::AUX, EpiTraits<EPI>::WARPS>::SMEM);
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
-  const cudaError_t e = launch_pdl(gemm_tc_kernel<BN, EPI>, dim3(grid), dim3(EpiTraits<EPI>::THREADS),
-                                   (size_t)TileCfg<BN, EpiTraits<EPI>::AUX, EpiTraits<EPI>::WARPS>::SMEM, st,
-                                   a, b, c, c2, x, p);
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = CG;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(grid * CG);
+  cfg.blockDim = dim3(E::THREADS);
+  cfg.dynamicSmemBytes = SMEM;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = CG == 2 ? 2 : 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k, a, b, c, c2, x, p);
   note_launch(1);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-template <int BN>
+template <int BN, int CG>
 cudaError_t dispatch(const CUtensorMap& a, const CUtensorMap& b, const CUtensorMap& c,
                      const CUtensorMap& c2, const CUtensorMap& x, const TcParams& p, int grid,
                      cudaStream_t st) {
   switch (p.epi) {
-    case EPI_STORE: return launch<BN, EPI_STORE>(a, b, c, c2, x, p, grid, st);
-    case EPI_BIAS_GELU: return launch<BN, EPI_BIAS_GELU>(a, b, c, c2, x, p, grid, st);
-    case EPI_MUL: return launch<BN, EPI_MUL>(a, b, c, c2, x, p, grid, st);
-    case EPI_BIAS_GELU_G: return launch<BN, EPI_BIAS_GELU_G>(a, b, c, c2, x, p, grid, st);
-    case EPI_RESID: return launch<BN, EPI_RESID>(a, b, c, c2, x, p, grid, st);
+    case EPI_STORE: return launch<BN, EPI_STORE, CG>(a, b, c, c2, x, p, grid, st);
+    case EPI_BIAS_GELU: return launch<BN, EPI_BIAS_GELU, CG>(a, b, c, c2, x, p, grid, st);
+    case EPI_MUL: return launch<BN, EPI_MUL, CG>(a, b, c, c2, x, p, grid, st);
+    case EPI_BIAS_GELU_G: return launch<BN, EPI_BIAS_GELU_G, CG>(a, b, c, c2, x, p, grid, st);
+    case EPI_RESID: return launch<BN, EPI_RESID, CG>(a, b, c, c2, x, p, grid, st);
     case EPI_SWIGLU:
     case EPI_DSWIGLU:
       // the gate|up epilogues work on 128-column blocks: 128- and 256-wide tiles only
       if constexpr (BN % 128 == 0) {
-        if (p.epi == EPI_SWIGLU) return launch<BN, EPI_SWIGLU>(a, b, c, c2, x, p, grid, st);
-        return launch<BN, EPI_DSWIGLU>(a, b, c, c2, x, p, grid, st);
+        if (p.epi == EPI_SWIGLU) return launch<BN, EPI_SWIGLU, CG>(a, b, c, c2, x, p, grid, st);
+        return launch<BN, EPI_DSWIGLU, CG>(a, b, c, c2, x, p, grid, st);
       }
       break;
   }
@@ -1018,22 +1106,36 @@ cudaError_t gemm_tc(const GemmArgs& g, cudaStream_t st) {
   const cudaError_t few = gemm_splitk(g, st);
   if (few != cudaErrorNotSupported) return few;
 
-  const int sms = device_sm_count();
-  const int m_tiles = (g.M + BM - 1) / BM;
-  // Tile width: fewest waves of 128 x BN tiles, weighted by each width's measured time per column
-  // and k-block (8192 x 3072 and 4096 x 3072, K = 768 and 1024: 0.22 us at 128 columns, 0.31 at
-  // 192, 0.365 at 256; the issue of the products and copies paces the narrow ones).  192 wins where
-  // it saves a wave or fills it (4096 x 768, K = 3072: 16.8 us against 19.1 at 256 and 22.9 at 128).
-  // Under the GELU epilogues the epilogue sets the pace and 192 costs no more per column than 256
-  // (8192 x 3072, K = 1024: 49.6 us at 192, 54.2 at 256; 4096 x 3072, K = 768: 29.7 and 31.0).
+  // Tile width, and one CTA or a pair to a tile, by the measured time of a launch: about 4.4 us (5.4
+  // for pairs: cluster barriers and the signals across them) plus waves x k-blocks x the time of a
+  // tile's k-block.  That is 0.222 us at 128 columns, 0.31 at 192 and 0.365 at 256 (8192 x 3072 and
+  // 4096 x 3072, K = 768 and 1024; the issue of the products and copies paces the narrow ones),
+  // 0.345 for a pair's 256 x 256 (half the operand bytes per product from L2: below 0.32 on long
+  // runs, more with the tile's start).  192 wins where it saves a wave or fills it (4096 x 768,
+  // K = 3072: 16.8 us against 19.1 at 256 and 22.9 at 128), pairs on several waves (8192 x 3072,
+  // K = 1024: 39 -> 34.3 us; 8192 x 1024, K = 4096: 46.5 -> 42.2; 8192 x 2048, K = 5632: 114.7 ->
+  // 100; but 8192 x 1024, K = 1024: 15.6, not 16.4; one wave is not short of L2: 4096 x 768,
+  // K = 3072: 17, not 20).  Under the GELU epilogues the epilogue sets the pace of short K: 192 costs
+  // no more per column than 256 (8192 x 3072, K = 1024: 49.6 us at 192, 54.2 at 256), and, as under
+  // the others that read an operand, pairs win from K of about 1536 (8192 x 1024, K = 3072 with GELU
+  // and GELU' 50.8 -> 41.5; 8192 x 4096, K = 1024: 64.4, not 69).
   const bool gelu = g.epi == EPI_BIAS_GELU || g.epi == EPI_BIAS_GELU_G;
-  auto cost = [&](int bn) {
-    int tiles = m_tiles * ((g.N + bn - 1) / bn);
-    int waves = (tiles + sms - 1) / sms;
-    return (double)waves * bn * (bn == 128 ? 1.22 : bn == 192 ? (gelu ? 0.99 : 1.14) : 1.0);
+  const int num_sms = device_sm_count(), kb = (g.K + BK - 1) / BK;
+  auto time_of = [&](int bn, int cg) {
+    const int tiles = ((g.M + BM * cg - 1) / (BM * cg)) * ((g.N + bn - 1) / bn), workers = num_sms / cg;
+    const int waves = (tiles + workers - 1) / workers;
+    const double per = cg == 2 ? 0.345 : bn == 128 ? 0.222 : bn == 192 ? (gelu ? 0.27 : 0.31) : 0.365;
+    return (cg == 2 ? 5.4 : 4.4) + (double)waves * kb * per;
   };
-  int BNsel = (g.N <= 128 || cost(128) < cost(256)) ? 128 : 256;
-  if (g.N > 128 && g.epi != EPI_SWIGLU && g.epi != EPI_DSWIGLU && cost(192) < cost(BNsel)) BNsel = 192;
+  int BNsel = (g.N <= 128 || time_of(128, 1) < time_of(256, 1)) ? 128 : 256;
+  if (g.N > 128 && g.epi != EPI_SWIGLU && g.epi != EPI_DSWIGLU && time_of(192, 1) < time_of(BNsel, 1)) BNsel = 192;
+  int cg = 1;
+  if ((g.epi == EPI_STORE || kb >= 24) && time_of(256, 2) < time_of(BNsel, 1)) {
+    BNsel = 256;
+    cg = 2;
+  }
+  const int sms = num_sms / cg;  // workers: CTAs, or pairs of them
+  const int m_tiles = (g.M + BM * cg - 1) / (BM * cg);
 
   CUtensorMap ma, mb, mc, mc2, mx;
   memset(&mc, 0, sizeof mc);
@@ -1043,9 +1145,9 @@ cudaError_t gemm_tc(const GemmArgs& g, cudaStream_t st) {
   // stored [K, N] B: one 3-D box per stage where N is a multiple of 64 (and the driver takes
   // the view), else BN / 64 boxes
   int b_kn = !g.b_kn ? 0 : g.N % 64 == 0 ? 2 : 1;
-  if (b_kn == 2 && !make_map(&mb, g.B, g.K, g.N, g.ldb, 64, BK, DT_BF16, BNsel / 64)) b_kn = 1;
+  if (b_kn == 2 && !make_map(&mb, g.B, g.K, g.N, g.ldb, 64, BK, DT_BF16, BNsel / cg / 64)) b_kn = 1;
   if (b_kn == 1 && !make_map(&mb, g.B, g.K, g.N, g.ldb, 64, BK, DT_BF16)) return cudaErrorNotSupported;
-  if (b_kn == 0 && !make_map(&mb, g.B, g.N, g.K, g.ldb, 64, BNsel, DT_BF16)) return cudaErrorNotSupported;
+  if (b_kn == 0 && !make_map(&mb, g.B, g.N, g.K, g.ldb, 64, BNsel / cg, DT_BF16)) return cudaErrorNotSupported;
   // output maps: C is [M, N] except the packed d(gate|up) output of the SwiGLU' epilogue,
   // [M, 2N]; C2 is [M, N] (bias+GELU) or [M, N / 2] (h of the SwiGLU epilogue)
   if (has_c) {
@@ -1094,7 +1196,7 @@ cudaError_t gemm_tc(const GemmArgs& g, cudaStream_t st) {
   p.sk_ws = g.sk_ws;
   p.sk_flags = g.sk_flags;
   const bool sk_epi = g.epi == EPI_STORE;
-  if (sk_epi && g.sk_ws && g.sk_flags && grid <= g.sk_slots && p.num_tiles > grid) {
+  if (sk_epi && g.sk_ws && g.sk_flags && grid * cg <= g.sk_slots && p.num_tiles > grid) {
     const int rem = p.num_tiles % grid;
     const long long iters = (long long)rem * p.k_blocks;
     const int ctas = (int)std::min<long long>(grid, iters / 8);
@@ -1104,9 +1206,10 @@ cudaError_t gemm_tc(const GemmArgs& g, cudaStream_t st) {
       p.sk_iters = (int)iters;
     }
   }
-  return BNsel == 256 ? dispatch<256>(ma, mb, mc, mc2, mx, p, grid, st)
-       : BNsel == 192 ? dispatch<192>(ma, mb, mc, mc2, mx, p, grid, st)
-                      : dispatch<128>(ma, mb, mc, mc2, mx, p, grid, st);
+  if (cg == 2) return dispatch<256, 2>(ma, mb, mc, mc2, mx, p, grid, st);
+  return BNsel == 256 ? dispatch<256, 1>(ma, mb, mc, mc2, mx, p, grid, st)
+       : BNsel == 192 ? dispatch<192, 1>(ma, mb, mc, mc2, mx, p, grid, st)
+                      : dispatch<128, 1>(ma, mb, mc, mc2, mx, p, grid, st);
 }
 
 }  // namespace ra
