@@ -76,17 +76,35 @@ __device__ __forceinline__ void load_a(uint32_t* a, const bf16* s, int ld, int r
   ldsm_x4(a, s + (size_t)r * ld + c);
 }
 
+// Each warp holds one k32 step's B fragments of up to eight n8 tiles (8 x 16 bytes a lane).  Where
+// the registers allow (AHEAD: up to 12 warps a CTA, at 85 a thread; at 64 they spill) each is
+// replaced as soon as its products are issued, so that the loads of the next step -- and, after the
+// last of phase 1, those of phase 2's first -- are in flight through the products, the z reduction
+// and the barriers, and the forward requests the first step's before pdl_wait: no kernel directly
+// before an adapter kernel writes its weights (the update is always further back), and at one
+// sequence of 128 tokens they come from DRAM.
+template <int MB>
+struct Phase1 {
+  static constexpr int NG = MB >= 64 ? MB / 64 : 1, NTG = MB >= 64 ? 8 : MB / 8;
+};
+template <int N>
+__device__ __forceinline__ void ld_frags(uint4 (&b)[8], const bf16* W, int C, int ntile, int k0, int lane) {
+#pragma unroll
+  for (int nt = 0; nt < N; ++nt) b[nt] = ld_frag2(W, C, ntile + nt, k0, lane);
+}
+
+constexpr bool ahead(int SZ) { return SZ == 0; }
+
 // Phase 1 shared by forward and backward: part[w] = X[16, kslice] * Bw^T over this warp's
 // slice [kbase, kbase + ks_len) of H, where Bw is [m, H] bf16 in the tiled fragment layout (B
-// fragments read directly, 16 bytes per thread per two k16 steps; the matrix is small and
-// stays in L1/L2).  The m output columns
-// are produced in groups of 8 n-tiles to bound the registers.  Rows of part are MB + 8 floats
-// apart, so the float2 stores of one half-warp fall in distinct banks.
-template <int MB>
-__device__ __forceinline__ void phase1_store(const bf16* Xs, int ldx, const bf16* Bw, int H,
+// fragments read directly, 16 bytes per thread per two k16 steps; AHEAD: b holds those of the first
+// step on entry).  The m output columns are produced in groups of 8 n-tiles to bound the registers.  Rows
+// of part are MB + 8 floats apart, so the float2 stores of one half-warp fall in distinct banks.
+template <int MB, bool AHEAD>
+__device__ __forceinline__ void phase1_store(uint4 (&b)[8], const bf16* Xs, int ldx, const bf16* Bw, int H,
                                              int kbase, int ks_len, float* part, int lane) {
   const int g = lane >> 2, t = lane & 3;
-  constexpr int NG = MB >= 64 ? MB / 64 : 1, NTG = MB >= 64 ? 8 : MB / 8;
+  constexpr int NG = Phase1<MB>::NG, NTG = Phase1<MB>::NTG;
 #pragma unroll 1
   for (int ng = 0; ng < NG; ++ng) {
     float acc[NTG][4];
@@ -94,14 +112,17 @@ __device__ __forceinline__ void phase1_store(const bf16* Xs, int ldx, const bf16
     for (int nt = 0; nt < NTG; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
 #pragma unroll 1
     for (int k0 = kbase; k0 < kbase + ks_len; k0 += 32) {
+      if (!AHEAD) ld_frags<NTG>(b, Bw, H, ng * 8, k0, lane);
       uint32_t a0[4], a1[4];
       load_a(a0, Xs, ldx, 0, k0, lane);
       load_a(a1, Xs, ldx, 0, k0 + 16, lane);
+      const bool wrap = k0 + 32 >= kbase + ks_len, more = !wrap || ng + 1 < NG;
+      const int kn = wrap ? kbase : k0 + 32, tn = (wrap ? ng + 1 : ng) * 8;
 #pragma unroll
       for (int nt = 0; nt < NTG; ++nt) {
-        const uint4 b = ld_frag2(Bw, H, ng * 8 + nt, k0, lane);
-        mma_bf16(acc[nt], a0, b.x, b.y);
-        mma_bf16(acc[nt], a1, b.z, b.w);
+        mma_bf16(acc[nt], a0, b[nt].x, b[nt].y);
+        mma_bf16(acc[nt], a1, b[nt].z, b[nt].w);
+        if (AHEAD && more) b[nt] = ld_frag2(Bw, H, tn + nt, kn, lane);
       }
     }
 #pragma unroll
@@ -120,24 +141,49 @@ __host__ __device__ inline int phase1_slice(int H, int m) {
 }
 
 // Phase 2: acc[16 rows, this warp's 64 columns] = S[16, m] * Bn^T where Bn is [H, m] bf16
-// in the tiled fragment layout (n = output column, k = bottleneck index).
-template <int MB>
-__device__ __forceinline__ void phase2(float (&acc)[8][4], const bf16* Ss, int lds,
+// in the tiled fragment layout (n = output column, k = bottleneck index); AHEAD: b holds the
+// fragments of its first step.
+template <int MB, bool AHEAD>
+__device__ __forceinline__ void phase2(uint4 (&b)[8], float (&acc)[8][4], const bf16* Ss, int lds,
                                        const bf16* Bn, int m, int nbase, int lane) {
 #pragma unroll
   for (int nt = 0; nt < 8; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
 #pragma unroll
   for (int k0 = 0; k0 < MB; k0 += 32) {
+    if (!AHEAD) ld_frags<8>(b, Bn, m, nbase >> 3, k0, lane);
     uint32_t a0[4], a1[4];
     load_a(a0, Ss, lds, 0, k0, lane);
     load_a(a1, Ss, lds, 0, k0 + 16, lane);
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) {
-      const uint4 b = ld_frag2(Bn, m, (nbase >> 3) + nt, k0, lane);
-      mma_bf16(acc[nt], a0, b.x, b.y);
-      mma_bf16(acc[nt], a1, b.z, b.w);
+      mma_bf16(acc[nt], a0, b[nt].x, b[nt].y);
+      mma_bf16(acc[nt], a1, b[nt].z, b[nt].w);
+      if (AHEAD && k0 + 32 < MB) b[nt] = ld_frag2(Bn, m, (nbase >> 3) + nt, k0 + 32, lane);
     }
   }
+}
+
+// Sum of the W1 warps' partials of z at row r, columns j .. j + 3 (four partials in flight; the
+// order is the warps')
+template <int MB>
+__device__ __forceinline__ float4 sum_partials(const float* part, int W1, int r, int j) {
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+  const float* p = part + r * (MB + 8) + j;
+  int w = 0;
+  for (; w + 4 <= W1; w += 4) {
+    float4 x[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) x[i] = *reinterpret_cast<const float4*>(p + (w + i) * R * (MB + 8));
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      s.x += x[i].x; s.y += x[i].y; s.z += x[i].z; s.w += x[i].w;
+    }
+  }
+  for (; w < W1; ++w) {
+    const float4 x = *reinterpret_cast<const float4*>(p + w * R * (MB + 8));
+    s.x += x.x; s.y += x.y; s.z += x.z; s.w += x.w;
+  }
+  return s;
 }
 
 struct FwdArgs {
@@ -246,8 +292,6 @@ template <int MB, int MODE, int SZ>
 __global__ void RA_ROWS_BOUNDS(SZ) adapter_fwd_mma_kernel(FwdArgs p) {
   constexpr bool DEC = MODE == FWD_RMS;
   extern __shared__ __align__(16) uint8_t sm[];
-  pdl_wait();
-  pdl_trigger();
   const int H = p.H, W = H / COLS_PER_WARP;
   const int KS = phase1_slice(H, MB), W1 = H / KS;
   const int lda = H + 8, lds = MB + 8;
@@ -263,7 +307,14 @@ __global__ void RA_ROWS_BOUNDS(SZ) adapter_fwd_mma_kernel(FwdArgs p) {
   const int t0 = blockIdx.x * R;
   const int nbase = warp * COLS_PER_WARP;
 
-  load_rows_bf16_async(As, lda, p.a, t0, p.T, H, R);
+  uint4 b[8];
+  if (ahead(SZ) && warp < W1) ld_frags<Phase1<MB>::NTG>(b, p.WdT, H, 0, warp * KS, lane);
+  if (blockIdx.x == 0) {  // the rest of the weights towards L2: they may come from DRAM
+    for (int e = threadIdx.x; e < H * MB / 64; e += blockDim.x) {
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(p.WdT + (size_t)e * 64));
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(p.WuT + (size_t)e * 64));
+    }
+  }
   if (p.stage_gb) {
     const int nv = (DEC ? 1 : 2) * (H / 4);
     for (int e = threadIdx.x; e < nv; e += blockDim.x) {
@@ -271,23 +322,27 @@ __global__ void RA_ROWS_BOUNDS(SZ) adapter_fwd_mma_kernel(FwdArgs p) {
       cp_async16(gbs + 4 * e, src, true);
     }
   }
+  pdl_wait();
+  pdl_trigger();
+  load_rows_bf16_async(As, lda, p.a, t0, p.T, H, R);
   cp_async_wait_all();
   __syncthreads();
-  if (warp < W1) phase1_store<MB>(As, lda, p.WdT, H, warp * KS, KS, part + (size_t)warp * R * (MB + 8), lane);
+  if (warp < W1) phase1_store<MB, ahead(SZ)>(b, As, lda, p.WdT, H, warp * KS, KS, part + (size_t)warp * R * (MB + 8), lane);
+  if (ahead(SZ)) ld_frags<8>(b, p.WuT, MB, nbase >> 3, 0, lane);
   __syncthreads();
-  for (int e = threadIdx.x; e < R * MB; e += blockDim.x) {
-    const int r = e / MB, j = e % MB;
-    float zs = 0.f;
-    for (int w = 0; w < W1; ++w) zs += part[((size_t)w * R + r) * (MB + 8) + j];
-    if (p.z && t0 + r < p.T) p.z[(size_t)(t0 + r) * MB + j] = zs;
-    Ss[r * lds + j] = __float2bfloat16_rn(gelu_f(zs));
+  for (int e = threadIdx.x; e < R * MB / 4; e += blockDim.x) {
+    const int r = e / (MB / 4), j = (e % (MB / 4)) * 4;
+    const float4 zs = sum_partials<MB>(part, W1, r, j);
+    if (p.z && t0 + r < p.T) *reinterpret_cast<float4*>(p.z + (size_t)(t0 + r) * MB + j) = zs;
+    *reinterpret_cast<uint2*>(Ss + r * lds + j) =
+        make_uint2(pack2(gelu_f(zs.x), gelu_f(zs.y)), pack2(gelu_f(zs.z), gelu_f(zs.w)));
   }
   __syncthreads();
   // encoder: the residual rows of this warp's columns land in the (now free) partial buffer
   // while phase 2 runs
   if (MODE == FWD_LN) load_block_async(Rs, lda, reinterpret_cast<const bf16*>(p.resid), t0, p.T, H, nbase, lane);
   float v[8][4];
-  phase2<MB>(v, Ss, lds, p.WuT, MB, nbase, lane);
+  phase2<MB, ahead(SZ)>(b, v, Ss, lds, p.WuT, MB, nbase, lane);
   if (MODE == FWD_LN) {
     cp_async_wait_all();
     __syncwarp();
@@ -339,8 +394,8 @@ __global__ void RA_ROWS_BOUNDS(SZ) adapter_fwd_mma_kernel(FwdArgs p) {
   s1 += __shfl_xor_sync(0xffffffffu, s1, 1);
   s1 += __shfl_xor_sync(0xffffffffu, s1, 2);
   // Row statistics with one barrier.  Each warp publishes a summary of its 64 columns of the
-  // 16 rows; after the barrier lanes 0-15 of every warp merge the W summaries of one row in
-  // warp order (the same order in every warp) and the quads fetch their two rows by shuffle.
+  // 16 rows; after the barrier two lanes of every warp merge the W summaries of one row, half each
+  // (the same order in every warp), and the quads fetch their two rows by shuffle.
   //   RMSNorm:   the sum of squares;
   //   LayerNorm: the mean and the centred sum of squares of the 64 columns, merged with the
   //              pairwise update of Chan, Golub and LeVeque for equal counts,
@@ -367,22 +422,32 @@ __global__ void RA_ROWS_BOUNDS(SZ) adapter_fwd_mma_kernel(FwdArgs p) {
   }
   __syncthreads();
   float mean = 0.f, rstd = 0.f;
-  if (lane < 16) {
+  {
+    const int rr = lane & 15, w0 = (lane >> 4) * ((W + 1) / 2), w1 = lane >> 4 ? W : (W + 1) / 2;
     if (DEC) {
       float q = 0.f;
-      for (int w = 0; w < W; ++w) q += stat[w * 16 + lane].y;
+#pragma unroll 4
+      for (int w = w0; w < w1; ++w) q += stat[w * 16 + rr].y;
+      q += __shfl_xor_sync(0xffffffffu, q, 16);
       rstd = rsqrtf(q / H + p.eps);
     } else {
-      float sm = 0.f;
-      for (int w = 0; w < W; ++w) sm += stat[w * 16 + lane].x;
-      mean = sm / W;
-      float q = 0.f, dd = 0.f;
-      for (int w = 0; w < W; ++w) {
-        const float2 st = stat[w * 16 + lane];
-        const float d = st.x - mean;
+      float sm = 0.f, q = 0.f;
+#pragma unroll 4
+      for (int w = w0; w < w1; ++w) {
+        const float2 st = stat[w * 16 + rr];
+        sm += st.x;
         q += st.y;
+      }
+      sm += __shfl_xor_sync(0xffffffffu, sm, 16);
+      q += __shfl_xor_sync(0xffffffffu, q, 16);
+      mean = sm / W;
+      float dd = 0.f;
+#pragma unroll 4
+      for (int w = w0; w < w1; ++w) {
+        const float d = stat[w * 16 + rr].x - mean;
         dd += d * d;
       }
+      dd += __shfl_xor_sync(0xffffffffu, dd, 16);
       rstd = rsqrtf((q + COLS_PER_WARP * dd) / H + p.eps);
     }
   }
@@ -443,8 +508,6 @@ struct BwdArgs {
 template <int MB, int SZ, bool DH_F32>
 __global__ void RA_ROWS_BOUNDS(SZ) adapter_bwd_rows_mma_kernel(BwdArgs p) {
   extern __shared__ __align__(16) uint8_t sm[];
-  pdl_wait();
-  pdl_trigger();
   const int H = p.H;
   const int KS = phase1_slice(H, MB), W1 = H / KS;
   const int ldg = H + 8, lds = MB + 8;
@@ -455,35 +518,40 @@ __global__ void RA_ROWS_BOUNDS(SZ) adapter_bwd_rows_mma_kernel(BwdArgs p) {
   const int g = lane >> 2, t = lane & 3;
   const int t0 = blockIdx.x * R;
 
+  const int nbase = warp * COLS_PER_WARP;
+  uint4 b[8];
+  pdl_wait();
+  pdl_trigger();
   load_rows_f32_as_bf16(Gs, ldg, p.g, t0, p.T, H, R);
+  if (ahead(SZ) && warp < W1) ld_frags<Phase1<MB>::NTG>(b, p.Wu, H, 0, warp * KS, lane);
   __syncthreads();
-  if (warp < W1) phase1_store<MB>(Gs, ldg, p.Wu, H, warp * KS, KS, part + (size_t)warp * R * (MB + 8), lane);
+  if (warp < W1) phase1_store<MB, ahead(SZ)>(b, Gs, ldg, p.Wu, H, warp * KS, KS, part + (size_t)warp * R * (MB + 8), lane);
+  if (ahead(SZ) && p.dh) ld_frags<8>(b, p.Wd, MB, nbase >> 3, 0, lane);
   __syncthreads();
   // the weight-gradient kernel reads GELU(z) and dz as the bf16 operands it multiplies: both
   // leave here rounded once, in the dz buffer ([T][m] GELU(z), then [T][m] dz)
   bf16* sz = reinterpret_cast<bf16*>(p.dz);
   bf16* dzb = sz + (size_t)p.T * MB;
-  for (int e = threadIdx.x; e < R * MB; e += blockDim.x) {
-    const int r = e / MB, j = e % MB;
-    float ds = 0.f;
-    for (int w = 0; w < W1; ++w) ds += part[((size_t)w * R + r) * (MB + 8) + j];
-    float dz = 0.f;
-    const bf16 d16 = __float2bfloat16_rn(0.f);
-    bf16 dzr = d16;
-    if (t0 + r < p.T) {
-      const float zz = p.z[(size_t)(t0 + r) * MB + j];
-      dz = ds * gelu_grad_f(zz);
-      dzr = __float2bfloat16_rn(dz);
-      sz[(size_t)(t0 + r) * MB + j] = __float2bfloat16_rn(gelu_f(zz));
-      dzb[(size_t)(t0 + r) * MB + j] = dzr;
+  for (int e = threadIdx.x; e < R * MB / 4; e += blockDim.x) {
+    const int r = e / (MB / 4), j = (e % (MB / 4)) * 4;
+    const bool live = t0 + r < p.T;
+    const size_t at = (size_t)(t0 + r) * MB + j;
+    float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (live) z = *reinterpret_cast<const float4*>(p.z + at);
+    const float4 ds = sum_partials<MB>(part, W1, r, j);
+    uint2 dz = make_uint2(0u, 0u);
+    if (live) {
+      dz = make_uint2(pack2(ds.x * gelu_grad_f(z.x), ds.y * gelu_grad_f(z.y)),
+                      pack2(ds.z * gelu_grad_f(z.z), ds.w * gelu_grad_f(z.w)));
+      *reinterpret_cast<uint2*>(sz + at) = make_uint2(pack2(gelu_f(z.x), gelu_f(z.y)), pack2(gelu_f(z.z), gelu_f(z.w)));
+      *reinterpret_cast<uint2*>(dzb + at) = dz;
     }
-    Ds[r * lds + j] = dzr;
+    *reinterpret_cast<uint2*>(Ds + r * lds + j) = dz;
   }
   if (!p.dh) return;
   __syncthreads();
-  const int nbase = warp * COLS_PER_WARP;
   float v[8][4];
-  phase2<MB>(v, Ds, lds, p.Wd, MB, nbase, lane);
+  phase2<MB, ahead(SZ)>(b, v, Ds, lds, p.Wd, MB, nbase, lane);
   const int r0 = t0 + g, r1 = r0 + 8;
   if (DH_F32) {
     // fp32 dh (the gradient feeding a LayerNorm backward), written from registers
