@@ -40,7 +40,7 @@ struct Cfg {
 };
 
 struct Params {
-  int M, N, k_blocks, b_kn, epi, split, m_tiles;
+  int M, N, k_blocks, b_kn, b_frozen, epi, split, m_tiles;
   void* C; int ldc; int c_dtype;
   const float* bias;
   void* C2; int ldc2; int c2_dtype;
@@ -117,31 +117,43 @@ __global__ void __launch_bounds__(THREADS, 1)
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_sh;
   cluster_arrive();  // (waited for before the first store to a peer: every CTA has then started)
-  // the set-up above overlaps the previous kernel's tail; operands are read only after it
-  pdl_wait();
-  pdl_trigger();
-
   const int S = p.split, rank = (int)cluster_rank();
   const int tile = blockIdx.x / S;
   const int m0 = (tile % p.m_tiles) * BM, n0 = (tile / p.m_tiles) * BN;
   const int kb0 = rank * p.k_blocks / S, kb1 = (rank + 1) * p.k_blocks / S;
 
+  // The set-up above overlaps the previous kernel's tail; a frozen B's first stages do too (at one
+  // sequence its weights come from DRAM, and the CTAs are mostly on idle SMs by then)
+  auto load_b = [&](int stage, int kb) {
+    const uint32_t sb = smem_base + stage * C::STAGE + C::A_BYTES;
+    if (p.b_kn) {
+#pragma unroll
+      for (int a = 0; a < BN / 64; ++a) tma_load_2d(&tmB, sb + a * 8192, &full_bar[stage], n0 + 64 * a, kb * BK);
+    } else {
+      tma_load_2d(&tmB, sb, &full_bar[stage], kb * BK, n0);
+    }
+  };
+  const int early = p.b_frozen ? min(STAGES, kb1 - kb0) : 0;
+  if (warp == 0 && elect_one())
+    for (int i = 0; i < early; ++i) {
+      mbar_expect_tx(&full_bar[i], C::STAGE);
+      load_b(i, kb0 + i);
+    }
+  __syncwarp();
+  pdl_wait();
+  pdl_trigger();
   if (warp == 0) {
     if (elect_one()) {
       int stage = 0, kb = kb0;
       uint32_t phase = 0;
       for (; kb < kb1; ++kb) {
-        if (!mbar_wait(&empty_bar[stage], phase ^ 1u, &abort_sh, p.err)) break;
-        mbar_expect_tx(&full_bar[stage], C::STAGE);
-        const uint32_t sa = smem_base + stage * C::STAGE;
-        tma_load_2d(&tmA, sa, &full_bar[stage], kb * BK, m0);
-        if (p.b_kn) {
-#pragma unroll
-          for (int a = 0; a < BN / 64; ++a)
-            tma_load_2d(&tmB, sa + C::A_BYTES + a * 8192, &full_bar[stage], n0 + 64 * a, kb * BK);
-        } else {
-          tma_load_2d(&tmB, sa + C::A_BYTES, &full_bar[stage], kb * BK, n0);
+        const bool b_here = kb - kb0 < early;
+        if (!b_here) {
+          if (!mbar_wait(&empty_bar[stage], phase ^ 1u, &abort_sh, p.err)) break;
+          mbar_expect_tx(&full_bar[stage], C::STAGE);
+          load_b(stage, kb);
         }
+        tma_load_2d(&tmA, smem_base + stage * C::STAGE, &full_bar[stage], kb * BK, m0);
         if (++stage == STAGES) { stage = 0; phase ^= 1u; }
       }
       if (kb < kb1) {  // given up: every copy that was started lands before the CTA goes away
@@ -352,7 +364,7 @@ cudaError_t gemm_splitk(const GemmArgs& g, cudaStream_t st) {
   if (g.b_kn ? !tma_map_bf16(&mb, g.B, g.K, g.N, g.ldb, 64, BK) : !tma_map_bf16(&mb, g.B, g.N, g.K, g.ldb, BK, bn))
     return cudaErrorNotSupported;
   Params p;
-  p.M = g.M; p.N = g.N; p.k_blocks = (g.K + BK - 1) / BK; p.b_kn = g.b_kn; p.epi = g.epi; p.split = split;
+  p.M = g.M; p.N = g.N; p.k_blocks = (g.K + BK - 1) / BK; p.b_kn = g.b_kn; p.b_frozen = g.b_frozen; p.epi = g.epi; p.split = split;
   p.m_tiles = (g.M + BM - 1) / BM;
   p.C = g.C; p.ldc = g.ldc; p.c_dtype = g.c_dtype; p.bias = g.bias;
   p.C2 = g.C2; p.ldc2 = g.ldc2; p.c2_dtype = g.c2_dtype;

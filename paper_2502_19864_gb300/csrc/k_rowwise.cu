@@ -65,6 +65,8 @@ int dw_chunks(int T, int H) {
 template <typename T>
 __global__ void layernorm_bwd_kernel(const float* dy, const float* dy2, const void* xhat, const float* rstd,
                                      const float* gamma, float* ds, void* ds_act, int Tn, int H) {
+  pdl_wait();
+  pdl_trigger();
   int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (t >= Tn) return;
   float s1 = 0.f, s2 = 0.f;
@@ -92,6 +94,8 @@ template <typename T>
 __global__ void add_layernorm_fwd_kernel(const void* x, const void* a, const float* gamma,
                                          const float* beta, float eps, void* y, void* xhat,
                                          float* rstd_out, int Tn, int H) {
+  pdl_wait();
+  pdl_trigger();
   int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (t >= Tn) return;
   const int64_t base = (int64_t)t * H;
@@ -115,6 +119,8 @@ __global__ void add_layernorm_fwd_kernel(const void* x, const void* a, const flo
 template <typename TX, typename TN>
 __global__ void rmsnorm_fwd_kernel(const void* x, const float* gamma, float eps, void* n,
                                    float* rstd, float* xf, int Tn, int H) {
+  pdl_wait();
+  pdl_trigger();
   int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (t >= Tn) return;
   float q = 0.f;
@@ -131,6 +137,8 @@ __global__ void rmsnorm_fwd_kernel(const void* x, const float* gamma, float eps,
 __global__ void rmsnorm_bwd_kernel(const float* dy, const float* x, const float* rstd,
                                    const float* gamma, const float* resid, float* dx, int Tn,
                                    int H) {
+  pdl_wait();
+  pdl_trigger();
   int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (t >= Tn) return;
   float s = 0.f;
@@ -331,6 +339,8 @@ template <typename T, int CM>
 __global__ void __launch_bounds__(HEAD_FWD_THREADS) encoder_head_fwd_kernel(const void* y, const float* Wh,
     const float* bh, const int32_t* labels, int B, int S, int H, int C, float* loss,
     float* logits_out, float* dlogits, unsigned* err) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ float lg[MAXB * MAXC];
   __shared__ float red[MAXB];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
@@ -415,6 +425,8 @@ __global__ void __launch_bounds__(HEAD_FWD_THREADS) encoder_head_fwd_kernel(cons
 template <typename T, int CM>
 __global__ void __launch_bounds__(HEAD_BWD_THREADS) encoder_head_bwd_kernel(const void* y, const float* Wh,
     const float* dlogits, int B, int S, int H, int C, float* dWh, float* dbh, float* dy) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ float lg[MAXB * MAXC];
   for (int e = threadIdx.x; e < B * C; e += blockDim.x) lg[e] = dlogits[e];
   __syncthreads();
@@ -547,6 +559,8 @@ __global__ void __launch_bounds__(64) span_head_ce_kernel(const int32_t* labels,
 // (a warp per token, 16-byte accesses; H % 4 == 0)
 __global__ void __launch_bounds__(256) span_head_dy_kernel(const float* Wh, const float* dlogits,
                                                            int Tn, int H, float* dy) {
+  pdl_wait();
+  pdl_trigger();
   const int64_t t = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (t >= Tn) return;
@@ -565,6 +579,8 @@ __global__ void __launch_bounds__(256) span_head_dy_kernel(const float* Wh, cons
 template <typename T>
 __global__ void __launch_bounds__(128) span_head_dw_kernel(const void* y, const float* dlogits,
     int Tn, int H, int chunk, float* part, float* part_b) {
+  pdl_wait();
+  pdl_trigger();
   const int i = blockIdx.x * 128 + threadIdx.x, c = blockIdx.y;
   const int t0 = c * chunk, t1 = min(Tn, t0 + chunk);
   if (i < H) {
@@ -594,6 +610,8 @@ __global__ void __launch_bounds__(128) span_head_dw_kernel(const void* y, const 
 // fixed-order sum of the chunk partials: dWh [2, H], dbh [2]
 __global__ void __launch_bounds__(256) span_head_dw_reduce_kernel(const float* part, const float* part_b,
     int nch, int H, float* dWh, float* dbh) {
+  pdl_wait();
+  pdl_trigger();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (dWh && j < 2 * H) {
     float s = 0.f;
@@ -739,6 +757,8 @@ __global__ void __launch_bounds__(256) vocab_ce_any_kernel(void* logits, int ld,
 }
 
 __global__ void __launch_bounds__(256) mean_kernel(const float* v, int n, float* out) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ float red[256];
   float s = 0.f;
   for (int i = threadIdx.x; i < n; i += 256) s += v[i];
@@ -759,6 +779,8 @@ __global__ void __launch_bounds__(256) mean_kernel(const float* v, int n, float*
 // element dominated the kernel's instructions); only a segment shorter than a block, lying
 // strictly inside one, falls back to evaluating them per element.
 __global__ void adam_kernel(AdamArgs a) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ float corr[2][2];  // [first / second segment of the block][lr / bc1, 1 / sqrt(bc2)]
   __shared__ int segs[2];
   const int64_t base = (int64_t)blockIdx.x * blockDim.x;
@@ -794,6 +816,8 @@ __global__ void adam_kernel(AdamArgs a) {
 }
 
 __global__ void bump_kernel(int32_t* steps, int n) {
+  pdl_wait();
+  pdl_trigger();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) steps[i] += 1;
 }
@@ -809,6 +833,8 @@ __global__ void convert_kernel(const float* src, void* dst, int64_t n) {
 
 template <typename T>
 __global__ void transpose_kernel(const float* src, void* dst, int rows, int cols, int ld_dst) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ float tile[32][33];
   int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
   for (int y = threadIdx.y; y < 32; y += 8) {
@@ -901,6 +927,8 @@ __global__ void __launch_bounds__(256) adapter_transpose_kernel(const float* P, 
 // correction per block.
 __global__ void __launch_bounds__(256) adam_adapter_kernel(AdamArgs a, float* PT, bf16* PB, bf16* PTB,
                                                            int H, int m) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ float tile[32][33];
   const int layer = blockIdx.z >> 2, mat = blockIdx.z & 3;
   const int64_t base = (int64_t)layer * 4 * H * m + (int64_t)mat * H * m;
@@ -944,6 +972,8 @@ __global__ void activation_kernel(int which, const float* x, float* y, int64_t n
   const float v = x[i];
   y[i] = which == 0 ? gelu_f(v) : which == 1 ? gelu_grad_f(v) : which == 2 ? silu_f(v) : silu_grad_f(v);
 }
+
+__global__ void fence_kernel() {}
 
 __global__ void fill_kernel(float* dst, float v, int64_t n) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -993,9 +1023,9 @@ cudaError_t layernorm_bwd(const float* dy, const float* dy2, const void* xhat, c
     if (dtype == DT_BF16) RA_VEC_SWITCH(V, ((void)launch_pdl(layernorm_bwd_vec_kernel<bf16, VV>, dim3(grid), dim3(256), (size_t)0, st, dy, dy2, xhat, rstd, gamma, ds, ds_act, T, H)))
     else RA_VEC_SWITCH(V, ((void)launch_pdl(layernorm_bwd_vec_kernel<float, VV>, dim3(grid), dim3(256), (size_t)0, st, dy, dy2, xhat, rstd, gamma, ds, ds_act, T, H)))
   } else if (dtype == DT_BF16) {
-    layernorm_bwd_kernel<bf16><<<grid, 256, 0, st>>>(dy, dy2, xhat, rstd, gamma, ds, ds_act, T, H);
+    (void)launch_pdl(layernorm_bwd_kernel<bf16>, dim3(grid), dim3(256), (size_t)0, st, dy, dy2, xhat, rstd, gamma, ds, ds_act, T, H);
   } else {
-    layernorm_bwd_kernel<float><<<grid, 256, 0, st>>>(dy, dy2, xhat, rstd, gamma, ds, ds_act, T, H);
+    (void)launch_pdl(layernorm_bwd_kernel<float>, dim3(grid), dim3(256), (size_t)0, st, dy, dy2, xhat, rstd, gamma, ds, ds_act, T, H);
   }
   note_launch(1);
   return cudaGetLastError();
@@ -1009,9 +1039,9 @@ cudaError_t add_layernorm_fwd(const void* x, const void* a, const float* gamma, 
     if (dtype == DT_BF16) RA_VEC_SWITCH(V, ((void)launch_pdl(add_layernorm_fwd_vec_kernel<bf16, VV>, dim3(grid), dim3(256), (size_t)0, st, x, a, gamma, beta, eps, y, xhat, rstd, T, H)))
     else RA_VEC_SWITCH(V, ((void)launch_pdl(add_layernorm_fwd_vec_kernel<float, VV>, dim3(grid), dim3(256), (size_t)0, st, x, a, gamma, beta, eps, y, xhat, rstd, T, H)))
   } else if (dtype == DT_BF16) {
-    add_layernorm_fwd_kernel<bf16><<<grid, 256, 0, st>>>(x, a, gamma, beta, eps, y, xhat, rstd, T, H);
+    (void)launch_pdl(add_layernorm_fwd_kernel<bf16>, dim3(grid), dim3(256), (size_t)0, st, x, a, gamma, beta, eps, y, xhat, rstd, T, H);
   } else {
-    add_layernorm_fwd_kernel<float><<<grid, 256, 0, st>>>(x, a, gamma, beta, eps, y, xhat, rstd, T, H);
+    (void)launch_pdl(add_layernorm_fwd_kernel<float>, dim3(grid), dim3(256), (size_t)0, st, x, a, gamma, beta, eps, y, xhat, rstd, T, H);
   }
   note_launch(1);
   return cudaGetLastError();
@@ -1034,13 +1064,13 @@ cudaError_t rmsnorm_fwd(const void* x, int x_dtype, const float* gamma, float ep
     return cudaGetLastError();
   }
   if (x_dtype == DT_BF16 && n_dtype == DT_BF16)
-    rmsnorm_fwd_kernel<bf16, bf16><<<grid, 256, 0, st>>>(x, gamma, eps, n, rstd, x_f32_out, T, H);
+    (void)launch_pdl(rmsnorm_fwd_kernel<bf16, bf16>, dim3(grid), dim3(256), (size_t)0, st, x, gamma, eps, n, rstd, x_f32_out, T, H);
   else if (x_dtype == DT_F32 && n_dtype == DT_BF16)
-    rmsnorm_fwd_kernel<float, bf16><<<grid, 256, 0, st>>>(x, gamma, eps, n, rstd, x_f32_out, T, H);
+    (void)launch_pdl(rmsnorm_fwd_kernel<float, bf16>, dim3(grid), dim3(256), (size_t)0, st, x, gamma, eps, n, rstd, x_f32_out, T, H);
   else if (x_dtype == DT_BF16)
-    rmsnorm_fwd_kernel<bf16, float><<<grid, 256, 0, st>>>(x, gamma, eps, n, rstd, x_f32_out, T, H);
+    (void)launch_pdl(rmsnorm_fwd_kernel<bf16, float>, dim3(grid), dim3(256), (size_t)0, st, x, gamma, eps, n, rstd, x_f32_out, T, H);
   else
-    rmsnorm_fwd_kernel<float, float><<<grid, 256, 0, st>>>(x, gamma, eps, n, rstd, x_f32_out, T, H);
+    (void)launch_pdl(rmsnorm_fwd_kernel<float, float>, dim3(grid), dim3(256), (size_t)0, st, x, gamma, eps, n, rstd, x_f32_out, T, H);
   note_launch(1);
   return cudaGetLastError();
 }
@@ -1050,7 +1080,7 @@ cudaError_t rmsnorm_bwd(const float* dy, const float* x, const float* rstd, cons
   if (const int V = row_vec(H))
     RA_VEC_SWITCH(V, ((void)launch_pdl(rmsnorm_bwd_vec_kernel<VV>, dim3(blocks_for((int64_t)T * 32, 256)), dim3(256), (size_t)0, st, dy, x, rstd, gamma, resid, dx, T, H)))
   else
-    rmsnorm_bwd_kernel<<<blocks_for((int64_t)T * 32, 256), 256, 0, st>>>(dy, x, rstd, gamma, resid, dx, T, H);
+    (void)launch_pdl(rmsnorm_bwd_kernel, dim3(blocks_for((int64_t)T * 32, 256)), dim3(256), (size_t)0, st, dy, x, rstd, gamma, resid, dx, T, H);
   note_launch(1);
   return cudaGetLastError();
 }
@@ -1063,7 +1093,7 @@ cudaError_t encoder_head_fwd(const void* y, int dtype, const float* Wh, const fl
                                : C <= 8 ? encoder_head_fwd_kernel<bf16, 8> : encoder_head_fwd_kernel<bf16, MAXC>)
                             : (C <= 2 ? encoder_head_fwd_kernel<float, 2>
                                : C <= 8 ? encoder_head_fwd_kernel<float, 8> : encoder_head_fwd_kernel<float, MAXC>);
-  k<<<1, HEAD_FWD_THREADS, 0, st>>>(y, Wh, bh, labels, B, S, H, C, loss, logits_out, dlogits, err);
+  (void)launch_pdl(k, dim3(1), dim3(HEAD_FWD_THREADS), (size_t)0, st, y, Wh, bh, labels, B, S, H, C, loss, logits_out, dlogits, err);
   note_launch(1);
   return cudaGetLastError();
 }
@@ -1077,7 +1107,7 @@ cudaError_t encoder_head_bwd(const void* y, int dtype, const float* Wh, const fl
                                : C <= 8 ? encoder_head_bwd_kernel<bf16, 8> : encoder_head_bwd_kernel<bf16, MAXC>)
                             : (C <= 2 ? encoder_head_bwd_kernel<float, 2>
                                : C <= 8 ? encoder_head_bwd_kernel<float, 8> : encoder_head_bwd_kernel<float, MAXC>);
-  k<<<grid, HEAD_BWD_THREADS, 0, st>>>(y, Wh, dlogits, B, S, H, C, dWh, dbh, dy);
+  (void)launch_pdl(k, dim3(grid), dim3(HEAD_BWD_THREADS), (size_t)0, st, y, Wh, dlogits, B, S, H, C, dWh, dbh, dy);
   note_launch(1);
   return cudaGetLastError();
 }
@@ -1095,7 +1125,7 @@ cudaError_t span_head_fwd(const void* y, int dtype, const float* Wh, const float
   if (e != cudaSuccess) return e;
   e = launch_pdl(span_head_ce_kernel, dim3(B), dim3(64), (size_t)0, st, labels, B, S, row_loss, logits_out, dlogits, err);
   if (e != cudaSuccess) return e;
-  mean_kernel<<<1, 256, 0, st>>>(row_loss, B, loss);
+  (void)launch_pdl(mean_kernel, dim3(1), dim3(256), (size_t)0, st, row_loss, B, loss);
   note_launch(3);
   return cudaGetLastError();
 }
@@ -1105,7 +1135,7 @@ cudaError_t span_head_bwd(const void* y, int dtype, const float* Wh, const float
                           cudaStream_t st) {
   if (H % 4) return cudaErrorInvalidValue;
   const int T = B * S;
-  span_head_dy_kernel<<<blocks_for((int64_t)T, 8), 256, 0, st>>>(Wh, dlogits, T, H, dy);
+  (void)launch_pdl(span_head_dy_kernel, dim3(blocks_for((int64_t)T, 8)), dim3(256), (size_t)0, st, Wh, dlogits, T, H, dy);
   note_launch(1);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || (!dWh && !dbh)) return e;
@@ -1113,19 +1143,21 @@ cudaError_t span_head_bwd(const void* y, int dtype, const float* Wh, const float
   float* part_b = part + (size_t)SPAN_CHUNKS * 2 * H;
   dim3 grid(blocks_for(H, 128), SPAN_CHUNKS);
   if (dtype == DT_BF16)
-    span_head_dw_kernel<bf16><<<grid, 128, 0, st>>>(y, dlogits, T, H, chunk, part, part_b);
+    (void)launch_pdl(span_head_dw_kernel<bf16>, dim3(grid), dim3(128), (size_t)0, st, y, dlogits, T, H, chunk, part, part_b);
   else
-    span_head_dw_kernel<float><<<grid, 128, 0, st>>>(y, dlogits, T, H, chunk, part, part_b);
+    (void)launch_pdl(span_head_dw_kernel<float>, dim3(grid), dim3(128), (size_t)0, st, y, dlogits, T, H, chunk, part, part_b);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  span_head_dw_reduce_kernel<<<blocks_for((int64_t)2 * H, 256), 256, 0, st>>>(part, part_b, SPAN_CHUNKS, H, dWh, dbh);
+  (void)launch_pdl(span_head_dw_reduce_kernel, dim3(blocks_for((int64_t)2 * H, 256)), dim3(256), (size_t)0, st, part, part_b, SPAN_CHUNKS, H, dWh, dbh);
   note_launch(2);
   return cudaGetLastError();
 }
 
 namespace {
 // Rows of whole 16-byte vectors that fit the registers of 512 threads (32768 bf16 or 16384 fp32
-// logits) are read once; other widths, strides and alignments take the three-pass kernel.
+// logits) are read once; other widths, strides and alignments take the three-pass kernel.  Plain
+// launches: started under the vocabulary GEMM's tail the step of two LLaMA-shaped blocks took 5750 us
+// instead of 5675.
 template <typename T>
 void launch_vocab_ce(void* logits, int ld, const int32_t* labels, int Tn, int V, float* row_loss,
                      float* logits_out, unsigned* err, cudaStream_t st) {
@@ -1150,21 +1182,27 @@ cudaError_t vocab_ce(void* logits, int dtype, int ld, const int32_t* labels, int
   else launch_vocab_ce<float>(logits, ld, labels, T, V, row_loss, logits_out, err, st);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  mean_kernel<<<1, 256, 0, st>>>(row_loss, T, loss);
+  (void)launch_pdl(mean_kernel, dim3(1), dim3(256), (size_t)0, st, row_loss, T, loss);
   note_launch(2);
   return cudaGetLastError();
 }
 
 cudaError_t adam_update(const AdamArgs& a, cudaStream_t st) {
   if (a.n <= 0) return cudaSuccess;
-  adam_kernel<<<blocks_for(a.n, 256), 256, 0, st>>>(a);
+  (void)launch_pdl(adam_kernel, dim3(blocks_for(a.n, 256)), dim3(256), (size_t)0, st, a);
   note_launch(1);
   return cudaGetLastError();
 }
 
 cudaError_t adam_bump(int32_t* steps, int n, cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
-  bump_kernel<<<blocks_for(n, 128), 128, 0, st>>>(steps, n);
+  (void)launch_pdl(bump_kernel, dim3(blocks_for(n, 128)), dim3(128), (size_t)0, st, steps, n);
+  note_launch(1);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_fence(cudaStream_t st) {
+  fence_kernel<<<1, 32, 0, st>>>();
   note_launch(1);
   return cudaGetLastError();
 }
@@ -1180,8 +1218,8 @@ cudaError_t convert_f32(const float* src, void* dst, int dst_dtype, int64_t n, c
 cudaError_t transpose_f32(const float* src, void* dst, int dst_dtype, int rows, int cols,
                           int ld_dst, cudaStream_t st) {
   dim3 grid((cols + 31) / 32, (rows + 31) / 32), blk(32, 8);
-  if (dst_dtype == DT_BF16) transpose_kernel<bf16><<<grid, blk, 0, st>>>(src, dst, rows, cols, ld_dst);
-  else transpose_kernel<float><<<grid, blk, 0, st>>>(src, dst, rows, cols, ld_dst);
+  if (dst_dtype == DT_BF16) (void)launch_pdl(transpose_kernel<bf16>, dim3(grid), dim3(blk), (size_t)0, st, src, dst, rows, cols, ld_dst);
+  else (void)launch_pdl(transpose_kernel<float>, dim3(grid), dim3(blk), (size_t)0, st, src, dst, rows, cols, ld_dst);
   note_launch(1);
   return cudaGetLastError();
 }
@@ -1210,7 +1248,7 @@ cudaError_t adam_adapter_update(const AdamArgs& a, float* PT, void* PB, void* PT
                                 int H, int m, cudaStream_t st) {
   if (n_layers <= 0) return cudaSuccess;
   dim3 grid((unsigned)(((H + 31) / 32) * ((m + 31) / 32)), 1, 4 * n_layers);
-  adam_adapter_kernel<<<grid, 256, 0, st>>>(a, PT, reinterpret_cast<bf16*>(PB), reinterpret_cast<bf16*>(PTB),
+  (void)launch_pdl(adam_adapter_kernel, dim3(grid), dim3(256), (size_t)0, st, a, PT, reinterpret_cast<bf16*>(PB), reinterpret_cast<bf16*>(PTB),
                                             H, m);
   note_launch(1);
   return cudaGetLastError();

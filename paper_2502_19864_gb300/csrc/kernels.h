@@ -59,6 +59,9 @@ struct GemmArgs {
   // without a transposed copy
   const void* B = nullptr; int ldb = 0;
   bool b_kn = false;
+  // B is a frozen weight: no kernel that may still run when this one starts (the stream's previous
+  // one) writes it, so its copies may start before that kernel has finished
+  bool b_frozen = false;
   int M = 0, N = 0, K = 0;
   int in_dtype = DT_F32;
   int epi = EPI_STORE;
@@ -279,6 +282,9 @@ cudaError_t adam_adapter_update(const AdamArgs& a, float* PT, void* PB, void* PT
                                 int H, int m, cudaStream_t st);
 
 // Utilities
+// An empty kernel, launched after everything before it in the stream: what follows may start early
+// relative to it alone
+cudaError_t launch_fence(cudaStream_t st);
 cudaError_t convert_f32(const float* src, void* dst, int dst_dtype, int64_t n, cudaStream_t st);
 // dst[c * ld_dst + r] = src[r, c] (src rows x cols, f32) converted to dst_dtype
 cudaError_t transpose_f32(const float* src, void* dst, int dst_dtype, int rows, int cols,

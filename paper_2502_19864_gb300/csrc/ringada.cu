@@ -546,6 +546,8 @@ ra_status ra_set_weights(ra_ctx* ctx, const ra_tensor_desc* list, int32_t n, ra_
   // transposed and bf16 copies of the adapters the step's kernels read
   if (adapters_changed)
     CU(adapter_transpose(ctx->P(), ctx->PT(), ctx->PB(), ctx->PTB(), ctx->L, H, m, st));
+  else if (n > 0)
+    CU(launch_fence(st));  // the next GEMM may read a frozen weight before its predecessor ends
   // every parameter of the model present?
   bool all = true;
   for (int l = -1; l < ctx->L && all; ++l)
@@ -647,6 +649,7 @@ GemmArgs gemm_args(const ra_ctx* c, const void* A, int lda, const void* B, int l
   GemmArgs g;
   g.A = A; g.lda = lda; g.B = B; g.ldb = ldb; g.M = M; g.N = N; g.K = K;
   g.in_dtype = c->act;
+  g.b_frozen = true;  // (every B is; ra_set_weights ends in a kernel that writes none)
   g.err = c->ws<unsigned>(c->ws_err);
   if (c->act == DT_BF16) {
     g.sk_ws = c->ws<float>(c->ws_sks[sk]);
