@@ -265,7 +265,8 @@ __global__ void __launch_bounds__(THREADS, 1)
       }
       if (p.epi == EPI_STORE || (p.epi == EPI_BIAS_GELU && p.C)) store4(p.C, p.c_dtype, (size_t)m * p.ldc + n, v);
       if (p.epi == EPI_BIAS_GELU) {
-        store4(p.C2, p.c2_dtype, (size_t)m * p.ldc2 + n, make_float4(gelu_f(v.x), gelu_f(v.y), gelu_f(v.z), gelu_f(v.w)));
+        const float2 y0 = gelu2(make_float2(v.x, v.y)), y1 = gelu2(make_float2(v.z, v.w));
+        store4(p.C2, p.c2_dtype, (size_t)m * p.ldc2 + n, make_float4(y0.x, y0.y, y1.x, y1.y));
       } else if (p.epi == EPI_BIAS_GELU_G) {
         float2 y0, d0, y1, d1;
         gelu_both2(make_float2(v.x, v.y), y0, d0);

@@ -358,8 +358,7 @@ struct EpiIn {
   float bias[32];
 };
 
-// GELU of 8 values, kept out of line: the epilogue then carries one copy of its code instead
-// of one per element, which keeps the hot loop inside the instruction cache.
+// GELU of 8 values
 struct F8 {
   float v[8];
 };
@@ -372,7 +371,7 @@ __device__ __forceinline__ F8 gelu8(F8 x) {
   }
   return x;
 }
-// GELU(u) into x and GELU'(u) into d for 8 values, out of line for the same reason
+// GELU(u) into x and GELU'(u) into d for 8 values
 struct F8x2 {
   F8 y, d;
 };
@@ -1115,22 +1114,23 @@ cudaError_t gemm_tc(const GemmArgs& g, cudaStream_t st) {
   // K = 3072: 16.8 us against 19.1 at 256 and 22.9 at 128), pairs on several waves (8192 x 3072,
   // K = 1024: 39 -> 34.3 us; 8192 x 1024, K = 4096: 46.5 -> 42.2; 8192 x 2048, K = 5632: 114.7 ->
   // 100; but 8192 x 1024, K = 1024: 15.6, not 16.4; one wave is not short of L2: 4096 x 768,
-  // K = 3072: 17, not 20).  Under the GELU epilogues the epilogue sets the pace of short K: 192 costs
-  // no more per column than 256 (8192 x 3072, K = 1024: 49.6 us at 192, 54.2 at 256), and, as under
-  // the others that read an operand, pairs win from K of about 1536 (8192 x 1024, K = 3072 with GELU
-  // and GELU' 50.8 -> 41.5; 8192 x 4096, K = 1024: 64.4, not 69).
+  // K = 3072: 17, not 20).  Under the GELU epilogues the epilogue adds to a tile's time, most to the
+  // wide ones (0.25, 0.305, 0.41 and 0.34: 4096 x 3072, K = 768 with GELU and GELU': 25.6, 23.4, 23.7
+  // and 24.6 us; 8192 x 4096, K = 1024: 67.4, 62.7, 58.8 and 53.2).  Under it and under those that
+  // read an operand, pairs lose on a K below 1024.
   const bool gelu = g.epi == EPI_BIAS_GELU || g.epi == EPI_BIAS_GELU_G;
   const int num_sms = device_sm_count(), kb = (g.K + BK - 1) / BK;
   auto time_of = [&](int bn, int cg) {
     const int tiles = ((g.M + BM * cg - 1) / (BM * cg)) * ((g.N + bn - 1) / bn), workers = num_sms / cg;
     const int waves = (tiles + workers - 1) / workers;
-    const double per = cg == 2 ? 0.345 : bn == 128 ? 0.222 : bn == 192 ? (gelu ? 0.27 : 0.31) : 0.365;
+    const double per = gelu ? (cg == 2 ? 0.34 : bn == 128 ? 0.25 : bn == 192 ? 0.305 : 0.41)
+                            : (cg == 2 ? 0.345 : bn == 128 ? 0.222 : bn == 192 ? 0.31 : 0.365);
     return (cg == 2 ? 5.4 : 4.4) + (double)waves * kb * per;
   };
   int BNsel = (g.N <= 128 || time_of(128, 1) < time_of(256, 1)) ? 128 : 256;
   if (g.N > 128 && g.epi != EPI_SWIGLU && g.epi != EPI_DSWIGLU && time_of(192, 1) < time_of(BNsel, 1)) BNsel = 192;
   int cg = 1;
-  if ((g.epi == EPI_STORE || kb >= 24) && time_of(256, 2) < time_of(BNsel, 1)) {
+  if ((g.epi == EPI_STORE || kb >= 16) && time_of(256, 2) < time_of(BNsel, 1)) {
     BNsel = 256;
     cg = 2;
   }
