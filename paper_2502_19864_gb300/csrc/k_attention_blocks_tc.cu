@@ -101,9 +101,26 @@ __device__ __forceinline__ void mma_xb(uint32_t d, uint32_t x, uint32_t b, bool 
                 sdesc_mn_sw128(b + n * (BR * 128) + kk * 2048), idesc, (acc || kk > 0) ? 1u : 0u);
 }
 
+// D[128 x 64] = X^T[128 x 128] B[128 x 64]: the staging block transposed (A read MN-major: its M
+// along the block's columns, two 64-wide atoms, K = its rows), B a 128 x 64 block read MN-major
+__device__ __forceinline__ void mma_xtb(uint32_t d, uint32_t x, uint32_t b) {
+  constexpr uint32_t idesc = idesc_bf16_abmn(BR, 64);
+#pragma unroll
+  for (int kk = 0; kk < BR / 16; ++kk)
+    umma_bf16(d, sdesc_mn_sw128_lbo(x + kk * 2048, BR * 128), sdesc_mn_sw128(b + kk * 2048), idesc, kk > 0 ? 1u : 0u);
+}
+
 // blockIdx.x = (batch, head); blockIdx.y = role (0: key pass of key block blockIdx.z -> dK,
-// dV; 1: query pass of query block blockIdx.z -> dQ)
-template <int DH, bool CAUSAL, bool ROPE>
+// dV; 1: query pass of query block blockIdx.z -> dQ).
+//
+// FUSED (head dim 64, at most two blocks: the encoders' sequences to 256): key passes alone, the one
+// or two of a (batch, head) as a cluster.  dS^T in the staging block is dS read MN-major, so each
+// pair of blocks also gives its share of dQ_i = dS k_j, in the score columns of TMEM that dP has
+// left; a CTA takes the other CTA's query block first, keeps that share in registers (32 a thread),
+// and at the end the shares change sides through the staging blocks and are added.  The scores, their
+// exponentials and dP are then computed once instead of in both passes, which set the pace: 32 x 16
+// heads of 256 78.6 us (92 in two passes), 32 x 12 of 128 23.1 (28.4).
+template <int DH, bool CAUSAL, bool ROPE, bool FUSED>
 __global__ void __launch_bounds__(NTHR, DH == 64 ? 2 : 1) attn_bwd_tc_kernel(AttnArgs a) {
   using Pl = BwdPlan<DH>;
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -118,7 +135,7 @@ __global__ void __launch_bounds__(NTHR, DH == 64 ? 2 : 1) attn_bwd_tc_kernel(Att
   const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   const int quad = warp & 3, half = warp >> 2;  // TMEM lane quadrant; 64-column half of a block
   const int bh = blockIdx.x, b = bh / a.n_heads, hh = bh % a.n_heads;
-  const bool keys = blockIdx.y == 0;
+  const bool keys = FUSED || blockIdx.y == 0;
   const int blk = blockIdx.z;                   // this CTA's key (or query) block
   const int S = a.S, NB = (S + BR - 1) / BR;
   const int H = a.n_heads * DH, ld = 3 * H;
@@ -239,29 +256,11 @@ __global__ void __launch_bounds__(NTHR, DH == 64 ? 2 : 1) attn_bwd_tc_kernel(Att
       }
     }
   };
-  // f * (TMEM columns [col, col + DH) of this thread's row) -> bf16 at dst (the row's DH head
-  // columns) when the row is live; this thread takes the head dims [16 DH/64 * half ...) in
-  // rotate-half pairs (d, d + DH/2) so that the RoPE transpose has both members (rope: the
-  // row's position s).  Every lane runs the TMEM loads (warp-wide); only the stores depend
-  // on the row.
-  auto store_row = [&](uint32_t col, bf16* dst, float f, bool live, bool rope, int s) {
+  // f * the rotate-half pairs (lo, hi) of this thread's row -> bf16 at dst (the row's DH head columns)
+  // when the row is live, with the RoPE transpose at position s when rope
+  auto store_pairs = [&](float* lo, float* hi, bf16* dst, float f, bool live, bool rope, int s) {
     constexpr int HALFD = DH / 2, PER = HALFD / 2;  // pairs per thread: 16 (DH 64) or 32
     const int i0 = PER * half;
-    float lo[32], hi[32];
-    if (PER == 32) {
-      tmem_ld32(trow + col + i0, lo);
-      tmem_ld32(trow + col + HALFD + i0, hi);
-    } else {  // DH 64: pairs (i, i + 32), i in [16 half, 16 half + 16)
-      float t[32];
-      tmem_ld32(trow + col, t);           // dims 0..31
-      float u[32];
-      tmem_ld32(trow + col + 32, u);      // dims 32..63
-#pragma unroll
-      for (int k = 0; k < 16; ++k) {  // compile-time indices on both sides (no local memory)
-        lo[k] = half ? t[16 + k] : t[k];
-        hi[k] = half ? u[16 + k] : u[k];
-      }
-    }
     if (!live) return;
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
@@ -286,6 +285,41 @@ __global__ void __launch_bounds__(NTHR, DH == 64 ? 2 : 1) attn_bwd_tc_kernel(Att
                      pk2(hi[8 * g + 4], hi[8 * g + 5]), pk2(hi[8 * g + 6], hi[8 * g + 7]));
     }
   };
+  // f * (TMEM columns [col, col + DH) of this thread's row) -> bf16 at dst (the row's DH head
+  // columns) when the row is live; this thread takes the head dims [16 DH/64 * half ...) in
+  // rotate-half pairs (d, d + DH/2) so that the RoPE transpose has both members (rope: the
+  // row's position s).  Every lane runs the TMEM loads (warp-wide); only the stores depend
+  // on the row.
+  auto store_row = [&](uint32_t col, bf16* dst, float f, bool live, bool rope, int s) {
+    constexpr int HALFD = DH / 2, PER = HALFD / 2;  // pairs per thread: 16 (DH 64) or 32
+    const int i0 = PER * half;
+    float lo[32], hi[32];
+    if (PER == 32) {
+      tmem_ld32(trow + col + i0, lo);
+      tmem_ld32(trow + col + HALFD + i0, hi);
+    } else {  // DH 64: pairs (i, i + 32), i in [16 half, 16 half + 16)
+      float t[32];
+      tmem_ld32(trow + col, t);           // dims 0..31
+      float u[32];
+      tmem_ld32(trow + col + 32, u);      // dims 32..63
+#pragma unroll
+      for (int k = 0; k < 16; ++k) {  // compile-time indices on both sides (no local memory)
+        lo[k] = half ? t[16 + k] : t[k];
+        hi[k] = half ? u[16 + k] : u[k];
+      }
+    }
+    store_pairs(lo, hi, dst, f, live, rope, s);
+  };
+  // this thread's pairs of dS k_j (head dims [16 half, + 16) and the same + 32) from the score columns
+  float share[32];
+  auto load_share = [&](float* v) {
+    tmem_ld16(trow + Pl::C_S + 16 * half, v);
+    tmem_ld16(trow + Pl::C_S + 32 + 16 * half, v + 16);
+  };
+  if (FUSED) {
+#pragma unroll
+    for (int k = 0; k < 32; ++k) share[k] = 0.f;
+  }
   constexpr uint32_t ID128 = idesc_bf16(BR, BR);
 
   if (keys) {
@@ -294,7 +328,10 @@ __global__ void __launch_bounds__(NTHR, DH == 64 ? 2 : 1) attn_bwd_tc_kernel(Att
     load_block<DH>(sb + Pl::T0, qkv + H, ld, j * BR, S);       // k_j
     load_block<DH>(sb + Pl::T1, qkv + 2 * H, ld, j * BR, S);   // v_j
     const int i_first = CAUSAL ? j : 0;
-    for (int i = i_first; i < NB && ok; ++i) {
+    bool first = true;
+    for (int it = i_first; it < NB && ok; ++it) {
+      // (FUSED: the other CTA's query block first, then this one's own)
+      const int i = FUSED && NB == 2 && !(CAUSAL && j == 1) ? (it == 0 ? 1 - j : j) : it;
       load_block<DH>(sb + Pl::T2, qkv, ld, i * BR, S);         // q_i
       load_block<DH>(sb + Pl::T3, dO, H, i * BR, S);           // dO_i
       load_stats(i * BR);
@@ -310,7 +347,7 @@ __global__ void __launch_bounds__(NTHR, DH == 64 ? 2 : 1) attn_bwd_tc_kernel(Att
       softmax_to_x(j * BR, i * BR);  // P^T
       publish();
       if (warp == 0 && elect_one()) {  // dV_j += P^T dO_i; dP^T = v_j dO_i^T
-        mma_xb<DH>(tmem + Pl::C_A, sb + Pl::X, sb + Pl::T3, i > i_first);
+        mma_xb<DH>(tmem + Pl::C_A, sb + Pl::X, sb + Pl::T3, !first);
         mma_qk<DH>(tmem + Pl::C_S, sb + Pl::T1, sb + Pl::T3, ID128);
         umma_commit(&bar);
       }
@@ -319,12 +356,40 @@ __global__ void __launch_bounds__(NTHR, DH == 64 ? 2 : 1) attn_bwd_tc_kernel(Att
       if (!ok) break;
       ds_in_x();  // dS^T over P^T (dV has read it)
       publish();
-      if (warp == 0 && elect_one()) {  // dK_j += dS^T q_i
-        mma_xb<DH>(tmem + Pl::C_B, sb + Pl::X, sb + Pl::T2, i > i_first);
+      if (warp == 0 && elect_one()) {  // dK_j += dS^T q_i (and dS k_j, over dP)
+        mma_xb<DH>(tmem + Pl::C_B, sb + Pl::X, sb + Pl::T2, !first);
+        if (FUSED) mma_xtb(tmem + Pl::C_S, sb + Pl::X, sb + Pl::T0);
         umma_commit(&bar);
       }
       pending = true;
       wait_mma();
+      if (FUSED && i != j) load_share(share);
+      first = false;
+    }
+    if (FUSED) {
+      const int q = j * BR + row;
+      if (NB == 2) {
+        cluster_arrive();
+        cluster_wait();  // neither CTA's products read its staging block any more
+        // 16-byte chunk c of row r at c ^ (r & 15): eight rows' stores fall in distinct banks
+        const uint32_t peer = peer_addr(sb + Pl::X + row * 256, (uint32_t)(1 - j));
+#pragma unroll
+        for (int g = 0; g < 8; ++g) st_cluster4(peer + (((8 * half + g) ^ (row & 15)) << 4), share + 4 * g);
+        cluster_arrive();
+        cluster_wait();
+      }
+      if (ok) {
+        load_share(share);
+        if (NB == 2) {
+          const uint8_t* mine = smem + Pl::X + row * 256;
+#pragma unroll
+          for (int g = 0; g < 8; ++g) {
+            const float4 o = *reinterpret_cast<const float4*>(mine + (((8 * half + g) ^ (row & 15)) << 4));
+            share[4 * g] += o.x; share[4 * g + 1] += o.y; share[4 * g + 2] += o.z; share[4 * g + 3] += o.w;
+          }
+        }
+        store_pairs(share, share + 16, dqkv + (size_t)(q < S ? q : 0) * ld, a.scale, q < S, ROPE, q);  // dQ
+      }
     }
     if (ok) {
       const int kk = j * BR + row;
@@ -389,19 +454,38 @@ __global__ void __launch_bounds__(NTHR, DH == 64 ? 2 : 1) attn_bwd_tc_kernel(Att
   }
 }
 
-template <int DH, bool CAUSAL, bool ROPE>
+template <int DH, bool CAUSAL, bool ROPE, bool FUSED>
 cudaError_t launch_bwd_tc(const AttnArgs& a, cudaStream_t st) {
-  auto k = attn_bwd_tc_kernel<DH, CAUSAL, ROPE>;
-  static bool attr = false;
-  if (!attr) {
+  auto k = attn_bwd_tc_kernel<DH, CAUSAL, ROPE, FUSED>;
+  static bool attr_set = false;
+  if (!attr_set) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdPlan<DH>::BYTES);
     if (e != cudaSuccess) return e;
-    attr = true;
+    attr_set = true;
   }
   const int nb = (a.S + BR - 1) / BR;
-  cudaError_t e = launch_pdl(k, dim3(a.B * a.n_heads, 2, nb), dim3(NTHR), (size_t)BwdPlan<DH>::BYTES, st, a);
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = nb;
+  cfg.gridDim = dim3(a.B * a.n_heads, FUSED ? 1 : 2, nb);
+  cfg.blockDim = dim3(NTHR);
+  cfg.dynamicSmemBytes = BwdPlan<DH>::BYTES;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = FUSED ? 2 : 1;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, k, a);
   note_launch(1);
   return e != cudaSuccess ? e : cudaGetLastError();
+}
+template <int DH, bool CAUSAL, bool ROPE>
+cudaError_t dispatch_bwd_tc(const AttnArgs& a, cudaStream_t st) {
+  if constexpr (DH == 64)
+    if (a.S <= 2 * BR) return launch_bwd_tc<DH, CAUSAL, ROPE, true>(a, st);
+  return launch_bwd_tc<DH, CAUSAL, ROPE, false>(a, st);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -665,11 +749,11 @@ cudaError_t attention_bwd_tc(const AttnArgs& a, cudaStream_t st) {
   if (!attention_bwd_tc_ok(a)) return cudaErrorNotSupported;
   const bool rope = a.rope;  // q and k were rotated in place by the forward
   if (a.head_dim == 64) {
-    if (a.causal) return rope ? launch_bwd_tc<64, true, true>(a, st) : launch_bwd_tc<64, true, false>(a, st);
-    return rope ? launch_bwd_tc<64, false, true>(a, st) : launch_bwd_tc<64, false, false>(a, st);
+    if (a.causal) return rope ? dispatch_bwd_tc<64, true, true>(a, st) : dispatch_bwd_tc<64, true, false>(a, st);
+    return rope ? dispatch_bwd_tc<64, false, true>(a, st) : dispatch_bwd_tc<64, false, false>(a, st);
   }
-  if (a.causal) return rope ? launch_bwd_tc<128, true, true>(a, st) : launch_bwd_tc<128, true, false>(a, st);
-  return rope ? launch_bwd_tc<128, false, true>(a, st) : launch_bwd_tc<128, false, false>(a, st);
+  if (a.causal) return rope ? dispatch_bwd_tc<128, true, true>(a, st) : dispatch_bwd_tc<128, true, false>(a, st);
+  return rope ? dispatch_bwd_tc<128, false, true>(a, st) : dispatch_bwd_tc<128, false, false>(a, st);
 }
 
 }  // namespace ra

@@ -55,12 +55,6 @@ __device__ __forceinline__ void tma_load_2d(const CUtensorMap* tm, uint32_t dst,
       "l"(reinterpret_cast<uint64_t>(tm)), "r"(c0), "r"(c1), "r"(smem_u32(bar))
       : "memory");
 }
-__device__ __forceinline__ void st_peer(uint32_t addr, const float* v) {
-  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v[0]), "f"(v[1]), "f"(v[2]),
-               "f"(v[3])
-               : "memory");
-}
-
 // four consecutive values at element offset `at` of a bf16 or fp32 matrix
 __device__ __forceinline__ float4 load4(const void* p, int dt, size_t at) {
   if (dt == DT_F32) return *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(p) + at);
@@ -208,7 +202,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       float v[32];
       tmem_ld32(tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(half * (BN / 2) + c), v);
 #pragma unroll
-      for (int q = 0; q < 8; ++q) st_peer(dst + (c + 4 * q) * 4, v + 4 * q);
+      for (int q = 0; q < 8; ++q) st_cluster4(dst + (c + 4 * q) * 4, v + 4 * q);
     }
   }
   tc_fence_before();
