@@ -27,6 +27,8 @@
 // after the query when causal, get P = 0.  Every wait on an MMA commit is bounded (global
 // timer); on expiry the kernel records RA_DEVERR_TIMEOUT, lets its issued products finish,
 // frees TMEM and returns.
+#include <cuda.h>
+
 #include "common.cuh"
 #include "kernels.h"
 #include "tcgen05.cuh"
@@ -78,6 +80,19 @@ __device__ __forceinline__ void load_block(uint32_t dst, const bf16* base, int l
     cp_async16b(dst + (j >> 3) * (BR * 128) + swz(r, j & 7), base + (size_t)(ok ? g : 0) * ld + 8 * j, ok);
   }
 }
+// the same block by TMA: rows [row, row + 128) of a [tokens, columns] matrix from column col on, one
+// box per 64-wide atom.  Rows at or beyond S hold the next sequence's (zeros past the last token):
+// their probabilities are zero.
+template <int DH>
+__device__ __forceinline__ void tma_block(const CUtensorMap* tm, uint32_t dst, uint64_t* bar, int col, int row) {
+#pragma unroll
+  for (int n = 0; n < DH / 64; ++n)
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3}], [%4];" ::"r"(dst + n * (BR * 128)),
+        "l"(reinterpret_cast<uint64_t>(tm)), "r"(col + 64 * n), "r"(row), "r"(smem_u32(bar))
+        : "memory");
+}
 // D[128 x 128] = A B^T over K = DH (both K-major 128 x DH blocks)
 template <int DH>
 __device__ __forceinline__ void mma_qk(uint32_t d, uint32_t a, uint32_t b, uint32_t idesc) {
@@ -119,12 +134,13 @@ __device__ __forceinline__ void mma_xtb(uint32_t d, uint32_t x, uint32_t b) {
 // left; a CTA takes the other CTA's query block first, keeps that share in registers (32 a thread),
 // and at the end the shares change sides through the staging blocks and are added.  The scores, their
 // exponentials and dP are then computed once instead of in both passes, which set the pace: 32 x 16
-// heads of 256 78.6 us (92 in two passes), 32 x 12 of 128 23.1 (28.4).
+// heads of 256 76.9 us (92 in two passes), 32 x 12 of 128 22.7 (28.4).
 template <int DH, bool CAUSAL, bool ROPE, bool FUSED>
-__global__ void __launch_bounds__(NTHR, DH == 64 ? 2 : 1) attn_bwd_tc_kernel(AttnArgs a) {
+__global__ void __launch_bounds__(NTHR, DH == 64 ? 2 : 1) attn_bwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV,
+    const __grid_constant__ CUtensorMap tmDO, AttnArgs a) {
   using Pl = BwdPlan<DH>;
   extern __shared__ __align__(1024) uint8_t smem[];
-  __shared__ __align__(8) uint64_t bar;
+  __shared__ __align__(8) uint64_t bar, load_bar;
   __shared__ uint32_t tmem_sh;
   __shared__ volatile int abort_sh;
   const uint32_t sb = smem_u32(smem);
@@ -139,8 +155,6 @@ __global__ void __launch_bounds__(NTHR, DH == 64 ? 2 : 1) attn_bwd_tc_kernel(Att
   const int blk = blockIdx.z;                   // this CTA's key (or query) block
   const int S = a.S, NB = (S + BR - 1) / BR;
   const int H = a.n_heads * DH, ld = 3 * H;
-  const bf16* qkv = reinterpret_cast<const bf16*>(a.qkv) + (size_t)b * S * ld + hh * DH;
-  const bf16* dO = reinterpret_cast<const bf16*>(a.dO) + (size_t)b * S * H + hh * DH;
   bf16* dqkv = reinterpret_cast<bf16*>(a.dqkv) + (size_t)b * S * ld + hh * DH;
   const float* lse = a.lse + (size_t)bh * S;
   const float* Dv = a.Dscratch + (size_t)bh * S;
@@ -148,10 +162,36 @@ __global__ void __launch_bounds__(NTHR, DH == 64 ? 2 : 1) attn_bwd_tc_kernel(Att
   float* DD = reinterpret_cast<float*>(smem + Pl::DD);
   const float sl2 = a.scale * kLog2e;
 
-  if (tid == 0) {
-    mbar_init(&bar, 1);
-    abort_sh = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  constexpr uint32_t BLK_BYTES = BR * DH * 2;
+  // q, k or v (part 0, 1, 2) rows of block blk_, or dO's, into a block of shared memory
+  auto load_qkv = [&](uint32_t dst, int part, int blk_) {
+    tma_block<DH>(&tmQKV, dst, &load_bar, part * H + hh * DH, b * S + blk_ * BR);
+  };
+  auto load_do = [&](uint32_t dst, int blk_) { tma_block<DH>(&tmDO, dst, &load_bar, hh * DH, b * S + blk_ * BR); };
+  if (warp == 1) {
+    // this warp starts the first copies while warp 0 allocates TMEM (about 1200 cycles)
+    if (elect_one()) {
+      mbar_init(&bar, 1);
+      mbar_init(&load_bar, 1);
+      abort_sh = 0;
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      pdl_wait();
+      mbar_expect_tx(&load_bar, 4 * BLK_BYTES);
+      if (keys) {
+        const int i = FUSED && NB == 2 && !(CAUSAL && blk == 1) ? 1 - blk : CAUSAL ? blk : 0;
+        load_qkv(sb + Pl::T0, 1, blk);
+        load_qkv(sb + Pl::T1, 2, blk);
+        load_qkv(sb + Pl::T2, 0, i);
+        load_do(sb + Pl::T3, i);
+      } else {
+        load_qkv(sb + Pl::T0, 0, blk);
+        load_do(sb + Pl::T1, blk);
+        load_qkv(sb + Pl::T2, 1, 0);
+        load_qkv(sb + Pl::T3, 2, 0);
+      }
+    }
+    __syncwarp();
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_sh)),
@@ -175,8 +215,7 @@ __global__ void __launch_bounds__(NTHR, DH == 64 ? 2 : 1) attn_bwd_tc_kernel(Att
 
   // every thread waits for the last commit; then a uniform view of whether it arrived
   auto wait_mma = [&]() {
-    if (ok) {
-      mbar_wait(&bar, phase, &abort_sh, a.err);
+    if (ok && mbar_wait(&bar, phase, &abort_sh, a.err)) {
       phase ^= 1u;
       pending = false;
     }
@@ -193,9 +232,17 @@ __global__ void __launch_bounds__(NTHR, DH == 64 ? 2 : 1) attn_bwd_tc_kernel(Att
     __syncthreads();
     tc_fence_after();
   };
+  // every thread waits for the copies of this round; then a barrier as above
+  uint32_t load_phase = 0;
+  bool loading = true;  // a round of copies was started and not yet waited for
   auto copies_done = [&]() {
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    loading = true;
+    if (ok && mbar_wait(&load_bar, load_phase, &abort_sh, a.err)) {
+      load_phase ^= 1u;
+      loading = false;
+    }
+    publish();
+    ok = ok && abort_sh == 0;
   };
   auto load_stats = [&](int q0) {
     for (int r = tid; r < BR; r += NTHR) {
@@ -325,18 +372,19 @@ __global__ void __launch_bounds__(NTHR, DH == 64 ? 2 : 1) attn_bwd_tc_kernel(Att
   if (keys) {
     // ------------------------------------------------------------ key pass: dK_j, dV_j
     const int j = blk;
-    load_block<DH>(sb + Pl::T0, qkv + H, ld, j * BR, S);       // k_j
-    load_block<DH>(sb + Pl::T1, qkv + 2 * H, ld, j * BR, S);   // v_j
     const int i_first = CAUSAL ? j : 0;
     bool first = true;
     for (int it = i_first; it < NB && ok; ++it) {
       // (FUSED: the other CTA's query block first, then this one's own)
       const int i = FUSED && NB == 2 && !(CAUSAL && j == 1) ? (it == 0 ? 1 - j : j) : it;
-      load_block<DH>(sb + Pl::T2, qkv, ld, i * BR, S);         // q_i
-      load_block<DH>(sb + Pl::T3, dO, H, i * BR, S);           // dO_i
+      if (!first && warp == 1 && elect_one()) {
+        mbar_expect_tx(&load_bar, 2 * BLK_BYTES);
+        load_qkv(sb + Pl::T2, 0, i);  // q_i
+        load_do(sb + Pl::T3, i);      // dO_i
+      }
       load_stats(i * BR);
       copies_done();
-      publish();
+      if (!ok) break;
       if (warp == 0 && elect_one()) {  // S^T = k_j q_i^T
         mma_qk<DH>(tmem + Pl::C_S, sb + Pl::T0, sb + Pl::T2, ID128);
         umma_commit(&bar);
@@ -366,49 +414,47 @@ __global__ void __launch_bounds__(NTHR, DH == 64 ? 2 : 1) attn_bwd_tc_kernel(Att
       if (FUSED && i != j) load_share(share);
       first = false;
     }
-    if (FUSED) {
-      const int q = j * BR + row;
-      if (NB == 2) {
-        cluster_arrive();
-        cluster_wait();  // neither CTA's products read its staging block any more
-        // 16-byte chunk c of row r at c ^ (r & 15): eight rows' stores fall in distinct banks
-        const uint32_t peer = peer_addr(sb + Pl::X + row * 256, (uint32_t)(1 - j));
+    const int kk = j * BR + row;
+    bf16* dst = dqkv + (size_t)(kk < S ? kk : 0) * ld;
+    const bool swap = FUSED && NB == 2;
+    // (the stores of dV and dK cover the waits for the other CTA)
+    if (swap) cluster_arrive();
+    if (ok) store_row(Pl::C_A, dst + 2 * H, 1.f, kk < S, false, kk);  // dV
+    if (swap) {
+      cluster_wait();  // neither CTA's products read its staging block any more
+      // 16-byte chunk c of row r at c ^ (r & 15): eight rows' stores fall in distinct banks
+      const uint32_t peer = peer_addr(sb + Pl::X + row * 256, (uint32_t)(1 - j));
 #pragma unroll
-        for (int g = 0; g < 8; ++g) st_cluster4(peer + (((8 * half + g) ^ (row & 15)) << 4), share + 4 * g);
-        cluster_arrive();
-        cluster_wait();
-      }
-      if (ok) {
-        load_share(share);
-        if (NB == 2) {
-          const uint8_t* mine = smem + Pl::X + row * 256;
-#pragma unroll
-          for (int g = 0; g < 8; ++g) {
-            const float4 o = *reinterpret_cast<const float4*>(mine + (((8 * half + g) ^ (row & 15)) << 4));
-            share[4 * g] += o.x; share[4 * g + 1] += o.y; share[4 * g + 2] += o.z; share[4 * g + 3] += o.w;
-          }
-        }
-        store_pairs(share, share + 16, dqkv + (size_t)(q < S ? q : 0) * ld, a.scale, q < S, ROPE, q);  // dQ
-      }
+      for (int g = 0; g < 8; ++g) st_cluster4(peer + (((8 * half + g) ^ (row & 15)) << 4), share + 4 * g);
+      cluster_arrive();
     }
-    if (ok) {
-      const int kk = j * BR + row;
-      bf16* dst = dqkv + (size_t)(kk < S ? kk : 0) * ld;
-      store_row(Pl::C_A, dst + 2 * H, 1.f, kk < S, false, kk);      // dV
-      store_row(Pl::C_B, dst + H, a.scale, kk < S, ROPE, kk);       // dK
+    if (ok) store_row(Pl::C_B, dst + H, a.scale, kk < S, ROPE, kk);   // dK
+    if (swap) cluster_wait();
+    if (FUSED && ok) {
+      load_share(share);
+      if (swap) {
+        const uint8_t* mine = smem + Pl::X + row * 256;
+#pragma unroll
+        for (int g = 0; g < 8; ++g) {
+          const float4 o = *reinterpret_cast<const float4*>(mine + (((8 * half + g) ^ (row & 15)) << 4));
+          share[4 * g] += o.x; share[4 * g + 1] += o.y; share[4 * g + 2] += o.z; share[4 * g + 3] += o.w;
+        }
+      }
+      store_pairs(share, share + 16, dst, a.scale, kk < S, ROPE, kk);  // dQ
     }
   } else {
     // ------------------------------------------------------------ query pass: dQ_i
     const int i = blk;
-    load_block<DH>(sb + Pl::T0, qkv, ld, i * BR, S);           // q_i
-    load_block<DH>(sb + Pl::T1, dO, H, i * BR, S);             // dO_i
     load_stats(i * BR);
     const int j_end = CAUSAL ? i + 1 : NB;
     for (int j = 0; j < j_end && ok; ++j) {
-      load_block<DH>(sb + Pl::T2, qkv + H, ld, j * BR, S);     // k_j
-      load_block<DH>(sb + Pl::T3, qkv + 2 * H, ld, j * BR, S); // v_j
+      if (j > 0 && warp == 1 && elect_one()) {
+        mbar_expect_tx(&load_bar, 2 * BLK_BYTES);
+        load_qkv(sb + Pl::T2, 1, j);  // k_j
+        load_qkv(sb + Pl::T3, 2, j);  // v_j
+      }
       copies_done();
-      publish();
+      if (!ok) break;
       if (warp == 0 && elect_one()) {  // S = q_i k_j^T
         mma_qk<DH>(tmem + Pl::C_S, sb + Pl::T0, sb + Pl::T2, ID128);
         umma_commit(&bar);
@@ -440,10 +486,12 @@ __global__ void __launch_bounds__(NTHR, DH == 64 ? 2 : 1) attn_bwd_tc_kernel(Att
     }
   }
 
-  if (pending) {
-    // a wait gave up: let the issued products finish before TMEM is released
+  if (pending || loading) {
+    // a wait gave up: let the issued copies and products finish before shared memory and TMEM are
+    // released
     volatile int no_abort = 0;
-    mbar_wait(&bar, phase, &no_abort, nullptr);
+    if (pending) mbar_wait(&bar, phase, &no_abort, nullptr);
+    if (loading) mbar_wait(&load_bar, load_phase, &no_abort, nullptr);
   }
   tc_fence_before();
   __syncthreads();
@@ -477,7 +525,13 @@ cudaError_t launch_bwd_tc(const AttnArgs& a, cudaStream_t st) {
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = FUSED ? 2 : 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, k, a);
+  // qkv [B S, 3 H] and dO [B S, H] in boxes of 64 columns x 128 rows
+  const int H = a.n_heads * DH;
+  CUtensorMap mq, md;
+  if (!tma_map_bf16(&mq, a.qkv, (int64_t)a.B * a.S, 3LL * H, 3LL * H, 64, BR) ||
+      !tma_map_bf16(&md, a.dO, (int64_t)a.B * a.S, H, H, 64, BR))
+    return cudaErrorNotSupported;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, k, mq, md, a);
   note_launch(1);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -741,7 +795,8 @@ cudaError_t attention_fwd_blocks_tc(const AttnArgs& a, cudaStream_t st) {
 
 bool attention_bwd_tc_ok(const AttnArgs& a) {
   return a.dtype == DT_BF16 && (a.head_dim == 64 || a.head_dim == 128) && a.S >= 1 &&
-         (!a.rope || a.qk_rotated) && a.lse && a.Dscratch;
+         (!a.rope || a.qk_rotated) && a.lse && a.Dscratch &&
+         ((reinterpret_cast<uintptr_t>(a.qkv) | reinterpret_cast<uintptr_t>(a.dO)) & 15) == 0;
 }
 
 // expects D = rowsum(dO * O) in a.Dscratch and the forward's lse
