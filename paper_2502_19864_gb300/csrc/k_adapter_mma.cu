@@ -11,7 +11,7 @@
 //   backward  dz = (g W_up^T) * GELU'(z); dh = g + dz W_down^T;
 //   dW        per row-chunk partials of dW_up = GELU(z)^T g and dW_down^T = dz^T h, summed
 //             afterwards in a fixed order (deterministic).
-// CTA = 16 rows x H / 64 warps (64 registers per thread, two CTAs per SM up to H = 1024).
+// CTA = 16 or 32 rows x H / 64 warps (see RA_ROWS_BOUNDS).
 // Phase 1 (the reduction over H) splits K across warps in slices of 64 (128 when the
 // partial buffer would pass 64 KB) and sums the per-warp partials of z in a fixed order;
 // phase 2 gives each warp 64 of the H output columns; row statistics for the norm are
@@ -22,7 +22,7 @@
 namespace ra {
 namespace {
 
-constexpr int COLS_PER_WARP = 64, R = 16;
+constexpr int COLS_PER_WARP = 64;
 
 __device__ __forceinline__ void mma_bf16(float* d, const uint32_t* a, uint32_t b0, uint32_t b1) {
   asm volatile(
@@ -93,71 +93,91 @@ __device__ __forceinline__ void ld_frags(uint4 (&b)[8], const bf16* W, int C, in
   for (int nt = 0; nt < N; ++nt) b[nt] = ld_frag2(W, C, ntile + nt, k0, lane);
 }
 
-constexpr bool ahead(int SZ) { return SZ == 0; }
+constexpr bool ahead(int SZ, int MT) { return SZ == 0 || MT == 2; }
 
 // Phase 1 shared by forward and backward: part[w] = X[16, kslice] * Bw^T over this warp's
 // slice [kbase, kbase + ks_len) of H, where Bw is [m, H] bf16 in the tiled fragment layout (B
 // fragments read directly, 16 bytes per thread per two k16 steps; AHEAD: b holds those of the first
 // step on entry).  The m output columns are produced in groups of 8 n-tiles to bound the registers.  Rows
 // of part are MB + 8 floats apart, so the float2 stores of one half-warp fall in distinct banks.
-template <int MB, bool AHEAD>
+template <int MB, bool AHEAD, int MT>
 __device__ __forceinline__ void phase1_store(uint4 (&b)[8], const bf16* Xs, int ldx, const bf16* Bw, int H,
                                              int kbase, int ks_len, float* part, int lane) {
   const int g = lane >> 2, t = lane & 3;
   constexpr int NG = Phase1<MB>::NG, NTG = Phase1<MB>::NTG;
 #pragma unroll 1
   for (int ng = 0; ng < NG; ++ng) {
-    float acc[NTG][4];
+    float acc[MT][NTG][4];
 #pragma unroll
-    for (int nt = 0; nt < NTG; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
+    for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+      for (int nt = 0; nt < NTG; ++nt) acc[mt][nt][0] = acc[mt][nt][1] = acc[mt][nt][2] = acc[mt][nt][3] = 0.f;
 #pragma unroll 1
     for (int k0 = kbase; k0 < kbase + ks_len; k0 += 32) {
       if (!AHEAD) ld_frags<NTG>(b, Bw, H, ng * 8, k0, lane);
-      uint32_t a0[4], a1[4];
-      load_a(a0, Xs, ldx, 0, k0, lane);
-      load_a(a1, Xs, ldx, 0, k0 + 16, lane);
+      uint32_t a0[MT][4], a1[MT][4];
+#pragma unroll
+      for (int mt = 0; mt < MT; ++mt) {
+        load_a(a0[mt], Xs, ldx, 16 * mt, k0, lane);
+        load_a(a1[mt], Xs, ldx, 16 * mt, k0 + 16, lane);
+      }
       const bool wrap = k0 + 32 >= kbase + ks_len, more = !wrap || ng + 1 < NG;
       const int kn = wrap ? kbase : k0 + 32, tn = (wrap ? ng + 1 : ng) * 8;
 #pragma unroll
       for (int nt = 0; nt < NTG; ++nt) {
-        mma_bf16(acc[nt], a0, b[nt].x, b[nt].y);
-        mma_bf16(acc[nt], a1, b[nt].z, b[nt].w);
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt) {
+          mma_bf16(acc[mt][nt], a0[mt], b[nt].x, b[nt].y);
+          mma_bf16(acc[mt][nt], a1[mt], b[nt].z, b[nt].w);
+        }
         if (AHEAD && more) b[nt] = ld_frag2(Bw, H, tn + nt, kn, lane);
       }
     }
 #pragma unroll
-    for (int nt = 0; nt < NTG; ++nt) {
-      const int c = ng * 64 + nt * 8 + 2 * t;
-      *reinterpret_cast<float2*>(part + g * (MB + 8) + c) = make_float2(acc[nt][0], acc[nt][1]);
-      *reinterpret_cast<float2*>(part + (g + 8) * (MB + 8) + c) = make_float2(acc[nt][2], acc[nt][3]);
-    }
+    for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+      for (int nt = 0; nt < NTG; ++nt) {
+        const int c = ng * 64 + nt * 8 + 2 * t;
+        float* q = part + (16 * mt + g) * (MB + 8) + c;
+        *reinterpret_cast<float2*>(q) = make_float2(acc[mt][nt][0], acc[mt][nt][1]);
+        *reinterpret_cast<float2*>(q + 8 * (MB + 8)) = make_float2(acc[mt][nt][2], acc[mt][nt][3]);
+      }
   }
 }
 
 // K-slice of phase 1: 64 columns of H per warp unless the per-warp partials of z would pass
-// 64 KB of shared memory, then 128 (and only the first H / 128 warps take part)
-__host__ __device__ inline int phase1_slice(int H, int m) {
-  return (H / 64) * R * m * 4 > 65536 ? 128 : 64;
+// 64 KB of shared memory (150 KB for 32 rows, one CTA an SM), then 128 (and only the first H / 128
+// warps take part)
+__host__ __device__ inline int phase1_slice(int H, int m, int R) {
+  return R == 16 ? ((H / 64) * R * m * 4 > 65536 ? 128 : 64) : ((H / 64) * R * (m + 8) * 4 > 150000 ? 128 : 64);
 }
 
-// Phase 2: acc[16 rows, this warp's 64 columns] = S[16, m] * Bn^T where Bn is [H, m] bf16
+// Phase 2: acc[16 MT rows, this warp's 64 columns] = S[16 MT, m] * Bn^T where Bn is [H, m] bf16
 // in the tiled fragment layout (n = output column, k = bottleneck index); AHEAD: b holds the
 // fragments of its first step.
-template <int MB, bool AHEAD>
-__device__ __forceinline__ void phase2(uint4 (&b)[8], float (&acc)[8][4], const bf16* Ss, int lds,
+template <int MB, bool AHEAD, int MT>
+__device__ __forceinline__ void phase2(uint4 (&b)[8], float (&acc)[MT][8][4], const bf16* Ss, int lds,
                                        const bf16* Bn, int m, int nbase, int lane) {
 #pragma unroll
-  for (int nt = 0; nt < 8; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
+  for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+    for (int nt = 0; nt < 8; ++nt) acc[mt][nt][0] = acc[mt][nt][1] = acc[mt][nt][2] = acc[mt][nt][3] = 0.f;
 #pragma unroll
   for (int k0 = 0; k0 < MB; k0 += 32) {
     if (!AHEAD) ld_frags<8>(b, Bn, m, nbase >> 3, k0, lane);
-    uint32_t a0[4], a1[4];
-    load_a(a0, Ss, lds, 0, k0, lane);
-    load_a(a1, Ss, lds, 0, k0 + 16, lane);
+    uint32_t a0[MT][4], a1[MT][4];
+#pragma unroll
+    for (int mt = 0; mt < MT; ++mt) {
+      load_a(a0[mt], Ss, lds, 16 * mt, k0, lane);
+      load_a(a1[mt], Ss, lds, 16 * mt, k0 + 16, lane);
+    }
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) {
-      mma_bf16(acc[nt], a0, b[nt].x, b[nt].y);
-      mma_bf16(acc[nt], a1, b[nt].z, b[nt].w);
+#pragma unroll
+      for (int mt = 0; mt < MT; ++mt) {
+        mma_bf16(acc[mt][nt], a0[mt], b[nt].x, b[nt].y);
+        mma_bf16(acc[mt][nt], a1[mt], b[nt].z, b[nt].w);
+      }
       if (AHEAD && k0 + 32 < MB) b[nt] = ld_frag2(Bn, m, (nbase >> 3) + nt, k0 + 32, lane);
     }
   }
@@ -165,7 +185,7 @@ __device__ __forceinline__ void phase2(uint4 (&b)[8], float (&acc)[8][4], const 
 
 // Sum of the W1 warps' partials of z at row r, columns j .. j + 3 (four partials in flight; the
 // order is the warps')
-template <int MB>
+template <int MB, int R>
 __device__ __forceinline__ float4 sum_partials(const float* part, int W1, int r, int j) {
   float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
   const float* p = part + r * (MB + 8) + j;
@@ -237,7 +257,13 @@ __device__ __forceinline__ void load_rows_f32_as_bf16(bf16* dst, int ld, const f
 
 // Thread-count classes (H / 64 warps): SZ 0 for H <= 768 (two CTAs per SM at 85 registers),
 // SZ 1 for H <= 1024 (two CTAs per SM at 64), SZ 2 above (one CTA per SM, 64 registers).
-#define RA_ROWS_BOUNDS(SZ) __launch_bounds__((SZ) == 0 ? 384 : (SZ) == 1 ? 512 : 1024, (SZ) == 2 ? 1 : 2)
+//
+// MT = 2: 32 rows a CTA, one CTA an SM (168 or 128 registers), for H <= 1024 and batches that give
+// every SM more than one tile of 16.  The rows in flight on an SM are the same, but a weight fragment
+// is read once for them instead of twice: the 256 KB of fragments that every 16 rows of H = 1024 read
+// from L2 were more than twice the rows' own bytes.  RA_MT_FIGURES
+#define RA_ROWS_BOUNDS(SZ, MT) \
+  __launch_bounds__((SZ) == 0 ? 384 : (SZ) == 1 ? 512 : 1024, (SZ) == 2 || (MT) == 2 ? 1 : 2)
 __host__ __device__ constexpr int size_class(int H) { return H <= 768 ? 0 : H <= 1024 ? 1 : 2; }
 
 // Shared-memory layout of the forward kernel (byte offsets):
@@ -245,17 +271,17 @@ __host__ __device__ constexpr int size_class(int H) { return H <= 768 ? 0 : H <=
 //   [part, s)       per-warp partials of z [W1][R][MB + 8] f32; once z is summed (encoder) the
 //                   residual rows [R][H + 8] bf16, then xhat of each warp's columns
 //   [s, stat)       GELU(z) [R][MB + 8] bf16
-//   [stat, gb)      per-warp row summaries [W][16] float2
+//   [stat, gb)      per-warp row summaries [W][R] float2
 //   [gb, bytes)     gamma (and beta) staged at the start, when they fit without costing a CTA
 struct FwdLayout { int part, s, stat, gb, bytes; };
-__host__ __device__ inline FwdLayout fwd_layout(int H, int m, int gb_floats) {
-  const int W = H / COLS_PER_WARP, W1 = H / phase1_slice(H, m);
+__host__ __device__ inline FwdLayout fwd_layout(int H, int m, int gb_floats, int R) {
+  const int W = H / COLS_PER_WARP, W1 = H / phase1_slice(H, m, R);
   const int zpart = W1 * R * (m + 8) * 4, rows = R * (H + 8) * 2;
   FwdLayout L;
   L.part = rows;
   L.s = L.part + (zpart > rows ? zpart : rows);
   L.stat = L.s + R * (m + 8) * 2;
-  L.gb = L.stat + W * 16 * 8;
+  L.gb = L.stat + W * R * 8;
   L.bytes = L.gb + gb_floats * 4;
   return L;
 }
@@ -288,14 +314,15 @@ __device__ __forceinline__ void store_block(bf16* dst, int H, const bf16* src, i
 // GELU(a W_down) W_up, no residual operand, no norm)
 enum : int { FWD_LN = 0, FWD_RMS = 1, FWD_NONE = 2 };
 
-template <int MB, int MODE, int SZ>
-__global__ void RA_ROWS_BOUNDS(SZ) adapter_fwd_mma_kernel(FwdArgs p) {
-  constexpr bool DEC = MODE == FWD_RMS;
+template <int MB, int MODE, int SZ, int MT>
+__global__ void RA_ROWS_BOUNDS(SZ, MT) adapter_fwd_mma_kernel(FwdArgs p) {
+  constexpr bool DEC = MODE == FWD_RMS, AHEAD = ahead(SZ, MT);
+  constexpr int R = 16 * MT;
   extern __shared__ __align__(16) uint8_t sm[];
   const int H = p.H, W = H / COLS_PER_WARP;
-  const int KS = phase1_slice(H, MB), W1 = H / KS;
+  const int KS = phase1_slice(H, MB, R), W1 = H / KS;
   const int lda = H + 8, lds = MB + 8;
-  const FwdLayout L = fwd_layout(H, MB, 0);
+  const FwdLayout L = fwd_layout(H, MB, 0, R);
   bf16* As = reinterpret_cast<bf16*>(sm);
   float* part = reinterpret_cast<float*>(sm + L.part);
   bf16* Rs = reinterpret_cast<bf16*>(sm + L.part);
@@ -308,7 +335,7 @@ __global__ void RA_ROWS_BOUNDS(SZ) adapter_fwd_mma_kernel(FwdArgs p) {
   const int nbase = warp * COLS_PER_WARP;
 
   uint4 b[8];
-  if (ahead(SZ) && warp < W1) ld_frags<Phase1<MB>::NTG>(b, p.WdT, H, 0, warp * KS, lane);
+  if (AHEAD && warp < W1) ld_frags<Phase1<MB>::NTG>(b, p.WdT, H, 0, warp * KS, lane);
   if (blockIdx.x == 0) {  // the rest of the weights towards L2: they may come from DRAM
     for (int e = threadIdx.x; e < H * MB / 64; e += blockDim.x) {
       asm volatile("prefetch.global.L2 [%0];" ::"l"(p.WdT + (size_t)e * 64));
@@ -327,12 +354,12 @@ __global__ void RA_ROWS_BOUNDS(SZ) adapter_fwd_mma_kernel(FwdArgs p) {
   load_rows_bf16_async(As, lda, p.a, t0, p.T, H, R);
   cp_async_wait_all();
   __syncthreads();
-  if (warp < W1) phase1_store<MB, ahead(SZ)>(b, As, lda, p.WdT, H, warp * KS, KS, part + (size_t)warp * R * (MB + 8), lane);
-  if (ahead(SZ)) ld_frags<8>(b, p.WuT, MB, nbase >> 3, 0, lane);
+  if (warp < W1) phase1_store<MB, AHEAD, MT>(b, As, lda, p.WdT, H, warp * KS, KS, part + (size_t)warp * R * (MB + 8), lane);
+  if (AHEAD) ld_frags<8>(b, p.WuT, MB, nbase >> 3, 0, lane);
   __syncthreads();
   for (int e = threadIdx.x; e < R * MB / 4; e += blockDim.x) {
     const int r = e / (MB / 4), j = (e % (MB / 4)) * 4;
-    const float4 zs = sum_partials<MB>(part, W1, r, j);
+    const float4 zs = sum_partials<MB, R>(part, W1, r, j);
     if (p.z && t0 + r < p.T) *reinterpret_cast<float4*>(p.z + (size_t)(t0 + r) * MB + j) = zs;
     *reinterpret_cast<uint2*>(Ss + r * lds + j) =
         make_uint2(pack2(gelu_f(zs.x), gelu_f(zs.y)), pack2(gelu_f(zs.z), gelu_f(zs.w)));
@@ -340,155 +367,171 @@ __global__ void RA_ROWS_BOUNDS(SZ) adapter_fwd_mma_kernel(FwdArgs p) {
   __syncthreads();
   // encoder: the residual rows of this warp's columns land in the (now free) partial buffer
   // while phase 2 runs
-  if (MODE == FWD_LN) load_block_async(Rs, lda, reinterpret_cast<const bf16*>(p.resid), t0, p.T, H, nbase, lane);
-  float v[8][4];
-  phase2<MB, ahead(SZ)>(b, v, Ss, lds, p.WuT, MB, nbase, lane);
+  if (MODE == FWD_LN) {
+#pragma unroll
+    for (int mt = 0; mt < MT; ++mt)
+      load_block_async(Rs + 16 * mt * lda, lda, reinterpret_cast<const bf16*>(p.resid), t0 + 16 * mt, p.T, H, nbase, lane);
+  }
+  float v[MT][8][4];
+  phase2<MB, AHEAD, MT>(b, v, Ss, lds, p.WuT, MB, nbase, lane);
   if (MODE == FWD_LN) {
     cp_async_wait_all();
     __syncwarp();
   }
   if (MODE == FWD_NONE) {
     // y = a + GELU(z) W_up, through this warp's columns of the a rows
-    const int rl0 = g, rl1 = g + 8;
 #pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-      const int c = nbase + nt * 8 + 2 * t;
-      const float2 a0 = unpack2(*reinterpret_cast<const uint32_t*>(As + (size_t)rl0 * lda + c));
-      const float2 a1 = unpack2(*reinterpret_cast<const uint32_t*>(As + (size_t)rl1 * lda + c));
-      *reinterpret_cast<uint32_t*>(As + (size_t)rl0 * lda + c) = pack2(v[nt][0] + a0.x, v[nt][1] + a0.y);
-      *reinterpret_cast<uint32_t*>(As + (size_t)rl1 * lda + c) = pack2(v[nt][2] + a1.x, v[nt][3] + a1.y);
+    for (int mt = 0; mt < MT; ++mt) {
+      const int rl0 = 16 * mt + g, rl1 = rl0 + 8;
+#pragma unroll
+      for (int nt = 0; nt < 8; ++nt) {
+        const int c = nbase + nt * 8 + 2 * t;
+        const float2 a0 = unpack2(*reinterpret_cast<const uint32_t*>(As + (size_t)rl0 * lda + c));
+        const float2 a1 = unpack2(*reinterpret_cast<const uint32_t*>(As + (size_t)rl1 * lda + c));
+        *reinterpret_cast<uint32_t*>(As + (size_t)rl0 * lda + c) = pack2(v[mt][nt][0] + a0.x, v[mt][nt][1] + a0.y);
+        *reinterpret_cast<uint32_t*>(As + (size_t)rl1 * lda + c) = pack2(v[mt][nt][2] + a1.x, v[mt][nt][3] + a1.y);
+      }
     }
     __syncwarp();
-    store_block(p.y, H, As, lda, t0, p.T, nbase, lane);
+#pragma unroll
+    for (int mt = 0; mt < MT; ++mt) store_block(p.y, H, As + 16 * mt * lda, lda, t0 + 16 * mt, p.T, nbase, lane);
     return;
   }
-  const int rl0 = g, rl1 = g + 8;  // local rows of c0/c1 and c2/c3
-  const int r0 = t0 + rl0, r1 = t0 + rl1;
-  float s0 = 0.f, s1 = 0.f;
-#pragma unroll
-  for (int nt = 0; nt < 8; ++nt) {
-    const int c = nbase + nt * 8 + 2 * t;
-    float2 a0 = unpack2(*reinterpret_cast<const uint32_t*>(As + (size_t)rl0 * lda + c));
-    float2 a1 = unpack2(*reinterpret_cast<const uint32_t*>(As + (size_t)rl1 * lda + c));
-    float2 q0 = make_float2(0.f, 0.f), q1 = make_float2(0.f, 0.f);
-    if (DEC) {
-      const float* rs = reinterpret_cast<const float*>(p.resid);
-      if (r0 < p.T) q0 = *reinterpret_cast<const float2*>(rs + (size_t)r0 * H + c);
-      if (r1 < p.T) q1 = *reinterpret_cast<const float2*>(rs + (size_t)r1 * H + c);
-    } else {
-      q0 = unpack2(*reinterpret_cast<const uint32_t*>(Rs + (size_t)rl0 * lda + c));
-      q1 = unpack2(*reinterpret_cast<const uint32_t*>(Rs + (size_t)rl1 * lda + c));
-    }
-    v[nt][0] += a0.x + q0.x; v[nt][1] += a0.y + q0.y;
-    v[nt][2] += a1.x + q1.x; v[nt][3] += a1.y + q1.y;
-    if (DEC) {
-      s0 += v[nt][0] * v[nt][0] + v[nt][1] * v[nt][1];
-      s1 += v[nt][2] * v[nt][2] + v[nt][3] * v[nt][3];
-    } else {
-      s0 += v[nt][0] + v[nt][1];
-      s1 += v[nt][2] + v[nt][3];
-    }
-  }
-  s0 += __shfl_xor_sync(0xffffffffu, s0, 1);
-  s0 += __shfl_xor_sync(0xffffffffu, s0, 2);
-  s1 += __shfl_xor_sync(0xffffffffu, s1, 1);
-  s1 += __shfl_xor_sync(0xffffffffu, s1, 2);
   // Row statistics with one barrier.  Each warp publishes a summary of its 64 columns of the
-  // 16 rows; after the barrier two lanes of every warp merge the W summaries of one row, half each
-  // (the same order in every warp), and the quads fetch their two rows by shuffle.
+  // rows; after the barrier one lane (two for 16 rows, half the warps each) of every warp merges the W
+  // summaries of a row (the same order in every warp), and the quads fetch their rows by shuffle.
   //   RMSNorm:   the sum of squares;
   //   LayerNorm: the mean and the centred sum of squares of the 64 columns, merged with the
   //              pairwise update of Chan, Golub and LeVeque for equal counts,
   //              M2 = sum_w M2_w + 64 sum_w (mean_w - mean)^2.
-  float mu0 = 0.f, mu1 = 0.f;
-  if (!DEC) {
-    mu0 = s0 * (1.f / COLS_PER_WARP);
-    mu1 = s1 * (1.f / COLS_PER_WARP);
-    s0 = s1 = 0.f;
+#pragma unroll
+  for (int mt = 0; mt < MT; ++mt) {
+    const int rl0 = 16 * mt + g, rl1 = rl0 + 8;  // local rows of c0/c1 and c2/c3
+    const int r0 = t0 + rl0, r1 = t0 + rl1;
+    float s0 = 0.f, s1 = 0.f;
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) {
-      const float d0 = v[nt][0] - mu0, d1 = v[nt][1] - mu0, d2 = v[nt][2] - mu1, d3 = v[nt][3] - mu1;
-      s0 += d0 * d0 + d1 * d1;
-      s1 += d2 * d2 + d3 * d3;
+      const int c = nbase + nt * 8 + 2 * t;
+      float* x = v[mt][nt];
+      float2 a0 = unpack2(*reinterpret_cast<const uint32_t*>(As + (size_t)rl0 * lda + c));
+      float2 a1 = unpack2(*reinterpret_cast<const uint32_t*>(As + (size_t)rl1 * lda + c));
+      float2 q0 = make_float2(0.f, 0.f), q1 = make_float2(0.f, 0.f);
+      if (DEC) {
+        const float* rs = reinterpret_cast<const float*>(p.resid);
+        if (r0 < p.T) q0 = *reinterpret_cast<const float2*>(rs + (size_t)r0 * H + c);
+        if (r1 < p.T) q1 = *reinterpret_cast<const float2*>(rs + (size_t)r1 * H + c);
+      } else {
+        q0 = unpack2(*reinterpret_cast<const uint32_t*>(Rs + (size_t)rl0 * lda + c));
+        q1 = unpack2(*reinterpret_cast<const uint32_t*>(Rs + (size_t)rl1 * lda + c));
+      }
+      x[0] += a0.x + q0.x; x[1] += a0.y + q0.y;
+      x[2] += a1.x + q1.x; x[3] += a1.y + q1.y;
+      if (DEC) {
+        s0 += x[0] * x[0] + x[1] * x[1];
+        s1 += x[2] * x[2] + x[3] * x[3];
+      } else {
+        s0 += x[0] + x[1];
+        s1 += x[2] + x[3];
+      }
     }
     s0 += __shfl_xor_sync(0xffffffffu, s0, 1);
     s0 += __shfl_xor_sync(0xffffffffu, s0, 2);
     s1 += __shfl_xor_sync(0xffffffffu, s1, 1);
     s1 += __shfl_xor_sync(0xffffffffu, s1, 2);
-  }
-  if (t == 0) {
-    stat[warp * 16 + rl0] = make_float2(mu0, s0);
-    stat[warp * 16 + rl1] = make_float2(mu1, s1);
+    float mu0 = 0.f, mu1 = 0.f;
+    if (!DEC) {
+      mu0 = s0 * (1.f / COLS_PER_WARP);
+      mu1 = s1 * (1.f / COLS_PER_WARP);
+      s0 = s1 = 0.f;
+#pragma unroll
+      for (int nt = 0; nt < 8; ++nt) {
+        const float* x = v[mt][nt];
+        const float d0 = x[0] - mu0, d1 = x[1] - mu0, d2 = x[2] - mu1, d3 = x[3] - mu1;
+        s0 += d0 * d0 + d1 * d1;
+        s1 += d2 * d2 + d3 * d3;
+      }
+      s0 += __shfl_xor_sync(0xffffffffu, s0, 1);
+      s0 += __shfl_xor_sync(0xffffffffu, s0, 2);
+      s1 += __shfl_xor_sync(0xffffffffu, s1, 1);
+      s1 += __shfl_xor_sync(0xffffffffu, s1, 2);
+    }
+    if (t == 0) {
+      stat[warp * R + rl0] = make_float2(mu0, s0);
+      stat[warp * R + rl1] = make_float2(mu1, s1);
+    }
   }
   __syncthreads();
   float mean = 0.f, rstd = 0.f;
   {
-    const int rr = lane & 15, w0 = (lane >> 4) * ((W + 1) / 2), w1 = lane >> 4 ? W : (W + 1) / 2;
+    const int rr = lane & (R - 1), hf = lane / R;  // (R = 32: every lane a row of its own)
+    const int w0 = hf * ((W + 1) / 2), w1 = R == 32 || hf ? W : (W + 1) / 2;
+    auto both = [](float x) { return R == 32 ? x : x + __shfl_xor_sync(0xffffffffu, x, 16); };
     if (DEC) {
       float q = 0.f;
 #pragma unroll 4
-      for (int w = w0; w < w1; ++w) q += stat[w * 16 + rr].y;
-      q += __shfl_xor_sync(0xffffffffu, q, 16);
-      rstd = rsqrtf(q / H + p.eps);
+      for (int w = w0; w < w1; ++w) q += stat[w * R + rr].y;
+      rstd = rsqrtf(both(q) / H + p.eps);
     } else {
       float sm = 0.f, q = 0.f;
 #pragma unroll 4
       for (int w = w0; w < w1; ++w) {
-        const float2 st = stat[w * 16 + rr];
+        const float2 st = stat[w * R + rr];
         sm += st.x;
         q += st.y;
       }
-      sm += __shfl_xor_sync(0xffffffffu, sm, 16);
-      q += __shfl_xor_sync(0xffffffffu, q, 16);
-      mean = sm / W;
+      mean = both(sm) / W;
+      q = both(q);
       float dd = 0.f;
 #pragma unroll 4
       for (int w = w0; w < w1; ++w) {
-        const float d = stat[w * 16 + rr].x - mean;
+        const float d = stat[w * R + rr].x - mean;
         dd += d * d;
       }
-      dd += __shfl_xor_sync(0xffffffffu, dd, 16);
-      rstd = rsqrtf((q + COLS_PER_WARP * dd) / H + p.eps);
+      rstd = rsqrtf((q + COLS_PER_WARP * both(dd)) / H + p.eps);
     }
   }
-  const float rs0 = __shfl_sync(0xffffffffu, rstd, rl0), rs1 = __shfl_sync(0xffffffffu, rstd, rl1);
   const float* gam = p.stage_gb ? gbs : p.gamma;
-  if (DEC) {
+  const float* bet = p.stage_gb ? gbs + H : p.beta;
 #pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-      const int c = nbase + nt * 8 + 2 * t;
-      const float2 gm = *reinterpret_cast<const float2*>(gam + c);
-      if (r0 < p.T) *reinterpret_cast<float2*>(p.x_out + (size_t)r0 * H + c) = make_float2(v[nt][0], v[nt][1]);
-      if (r1 < p.T) *reinterpret_cast<float2*>(p.x_out + (size_t)r1 * H + c) = make_float2(v[nt][2], v[nt][3]);
-      // y goes through this warp's columns of the a rows (read above by this thread only)
-      *reinterpret_cast<uint32_t*>(As + (size_t)rl0 * lda + c) = pack2(v[nt][0] * rs0 * gm.x, v[nt][1] * rs0 * gm.y);
-      *reinterpret_cast<uint32_t*>(As + (size_t)rl1 * lda + c) = pack2(v[nt][2] * rs1 * gm.x, v[nt][3] * rs1 * gm.y);
+  for (int mt = 0; mt < MT; ++mt) {
+    const int rl0 = 16 * mt + g, rl1 = rl0 + 8, r0 = t0 + rl0, r1 = t0 + rl1;
+    const float rs0 = __shfl_sync(0xffffffffu, rstd, rl0), rs1 = __shfl_sync(0xffffffffu, rstd, rl1);
+    if (DEC) {
+#pragma unroll
+      for (int nt = 0; nt < 8; ++nt) {
+        const int c = nbase + nt * 8 + 2 * t;
+        const float* x = v[mt][nt];
+        const float2 gm = *reinterpret_cast<const float2*>(gam + c);
+        if (r0 < p.T) *reinterpret_cast<float2*>(p.x_out + (size_t)r0 * H + c) = make_float2(x[0], x[1]);
+        if (r1 < p.T) *reinterpret_cast<float2*>(p.x_out + (size_t)r1 * H + c) = make_float2(x[2], x[3]);
+        // y goes through this warp's columns of the a rows (read above by this thread only)
+        *reinterpret_cast<uint32_t*>(As + (size_t)rl0 * lda + c) = pack2(x[0] * rs0 * gm.x, x[1] * rs0 * gm.y);
+        *reinterpret_cast<uint32_t*>(As + (size_t)rl1 * lda + c) = pack2(x[2] * rs1 * gm.x, x[3] * rs1 * gm.y);
+      }
+    } else {
+      const float m0 = __shfl_sync(0xffffffffu, mean, rl0), m1 = __shfl_sync(0xffffffffu, mean, rl1);
+#pragma unroll
+      for (int nt = 0; nt < 8; ++nt) {
+        const int c = nbase + nt * 8 + 2 * t;
+        const float* x = v[mt][nt];
+        const float2 gm = *reinterpret_cast<const float2*>(gam + c);
+        const float2 bt = *reinterpret_cast<const float2*>(bet + c);
+        const float x00 = (x[0] - m0) * rs0, x01 = (x[1] - m0) * rs0;
+        const float x10 = (x[2] - m1) * rs1, x11 = (x[3] - m1) * rs1;
+        // y and xhat go through this warp's columns of the a rows and of the residual rows
+        *reinterpret_cast<uint32_t*>(As + (size_t)rl0 * lda + c) = pack2(x00 * gm.x + bt.x, x01 * gm.y + bt.y);
+        *reinterpret_cast<uint32_t*>(As + (size_t)rl1 * lda + c) = pack2(x10 * gm.x + bt.x, x11 * gm.y + bt.y);
+        *reinterpret_cast<uint32_t*>(Rs + (size_t)rl0 * lda + c) = pack2(x00, x01);
+        *reinterpret_cast<uint32_t*>(Rs + (size_t)rl1 * lda + c) = pack2(x10, x11);
+      }
     }
     __syncwarp();
-    store_block(p.y, H, As, lda, t0, p.T, nbase, lane);
-  } else {
-    const float m0 = __shfl_sync(0xffffffffu, mean, rl0), m1 = __shfl_sync(0xffffffffu, mean, rl1);
-    const float* bet = p.stage_gb ? gbs + H : p.beta;
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-      const int c = nbase + nt * 8 + 2 * t;
-      const float2 gm = *reinterpret_cast<const float2*>(gam + c);
-      const float2 bt = *reinterpret_cast<const float2*>(bet + c);
-      const float x00 = (v[nt][0] - m0) * rs0, x01 = (v[nt][1] - m0) * rs0;
-      const float x10 = (v[nt][2] - m1) * rs1, x11 = (v[nt][3] - m1) * rs1;
-      // y and xhat go through this warp's columns of the a rows and of the residual rows
-      *reinterpret_cast<uint32_t*>(As + (size_t)rl0 * lda + c) = pack2(x00 * gm.x + bt.x, x01 * gm.y + bt.y);
-      *reinterpret_cast<uint32_t*>(As + (size_t)rl1 * lda + c) = pack2(x10 * gm.x + bt.x, x11 * gm.y + bt.y);
-      *reinterpret_cast<uint32_t*>(Rs + (size_t)rl0 * lda + c) = pack2(x00, x01);
-      *reinterpret_cast<uint32_t*>(Rs + (size_t)rl1 * lda + c) = pack2(x10, x11);
+    store_block(p.y, H, As + 16 * mt * lda, lda, t0 + 16 * mt, p.T, nbase, lane);
+    if (!DEC && p.xhat) store_block(p.xhat, H, Rs + 16 * mt * lda, lda, t0 + 16 * mt, p.T, nbase, lane);
+    if (p.rstd && warp == 0 && t == 0) {
+      if (r0 < p.T) p.rstd[r0] = rs0;
+      if (r1 < p.T) p.rstd[r1] = rs1;
     }
-    __syncwarp();
-    store_block(p.y, H, As, lda, t0, p.T, nbase, lane);
-    if (p.xhat) store_block(p.xhat, H, Rs, lda, t0, p.T, nbase, lane);
-  }
-  if (p.rstd && warp == 0 && t == 0) {
-    if (r0 < p.T) p.rstd[r0] = rs0;
-    if (r1 < p.T) p.rstd[r1] = rs1;
   }
 }
 
@@ -505,11 +548,13 @@ struct BwdArgs {
   void* dh;           // [T, H] or null: bf16, or f32 when DH_F32
 };
 
-template <int MB, int SZ, bool DH_F32>
-__global__ void RA_ROWS_BOUNDS(SZ) adapter_bwd_rows_mma_kernel(BwdArgs p) {
+template <int MB, int SZ, bool DH_F32, int MT>
+__global__ void RA_ROWS_BOUNDS(SZ, MT) adapter_bwd_rows_mma_kernel(BwdArgs p) {
   extern __shared__ __align__(16) uint8_t sm[];
+  constexpr bool AHEAD = ahead(SZ, MT);
+  constexpr int R = 16 * MT;
   const int H = p.H;
-  const int KS = phase1_slice(H, MB), W1 = H / KS;
+  const int KS = phase1_slice(H, MB, R), W1 = H / KS;
   const int ldg = H + 8, lds = MB + 8;
   bf16* Gs = reinterpret_cast<bf16*>(sm);
   float* part = reinterpret_cast<float*>(Gs + (size_t)R * ldg);
@@ -523,10 +568,10 @@ __global__ void RA_ROWS_BOUNDS(SZ) adapter_bwd_rows_mma_kernel(BwdArgs p) {
   pdl_wait();
   pdl_trigger();
   load_rows_f32_as_bf16(Gs, ldg, p.g, t0, p.T, H, R);
-  if (ahead(SZ) && warp < W1) ld_frags<Phase1<MB>::NTG>(b, p.Wu, H, 0, warp * KS, lane);
+  if (AHEAD && warp < W1) ld_frags<Phase1<MB>::NTG>(b, p.Wu, H, 0, warp * KS, lane);
   __syncthreads();
-  if (warp < W1) phase1_store<MB, ahead(SZ)>(b, Gs, ldg, p.Wu, H, warp * KS, KS, part + (size_t)warp * R * (MB + 8), lane);
-  if (ahead(SZ) && p.dh) ld_frags<8>(b, p.Wd, MB, nbase >> 3, 0, lane);
+  if (warp < W1) phase1_store<MB, AHEAD, MT>(b, Gs, ldg, p.Wu, H, warp * KS, KS, part + (size_t)warp * R * (MB + 8), lane);
+  if (AHEAD && p.dh) ld_frags<8>(b, p.Wd, MB, nbase >> 3, 0, lane);
   __syncthreads();
   // the weight-gradient kernel reads GELU(z) and dz as the bf16 operands it multiplies: both
   // leave here rounded once, in the dz buffer ([T][m] GELU(z), then [T][m] dz)
@@ -538,7 +583,7 @@ __global__ void RA_ROWS_BOUNDS(SZ) adapter_bwd_rows_mma_kernel(BwdArgs p) {
     const size_t at = (size_t)(t0 + r) * MB + j;
     float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
     if (live) z = *reinterpret_cast<const float4*>(p.z + at);
-    const float4 ds = sum_partials<MB>(part, W1, r, j);
+    const float4 ds = sum_partials<MB, R>(part, W1, r, j);
     uint2 dz = make_uint2(0u, 0u);
     if (live) {
       dz = make_uint2(pack2(ds.x * gelu_grad_f(z.x), ds.y * gelu_grad_f(z.y)),
@@ -550,38 +595,43 @@ __global__ void RA_ROWS_BOUNDS(SZ) adapter_bwd_rows_mma_kernel(BwdArgs p) {
   }
   if (!p.dh) return;
   __syncthreads();
-  float v[8][4];
-  phase2<MB, ahead(SZ)>(b, v, Ds, lds, p.Wd, MB, nbase, lane);
-  const int r0 = t0 + g, r1 = r0 + 8;
-  if (DH_F32) {
-    // fp32 dh (the gradient feeding a LayerNorm backward), written from registers
-    float* dh = reinterpret_cast<float*>(p.dh);
+  float v[MT][8][4];
+  phase2<MB, AHEAD, MT>(b, v, Ds, lds, p.Wd, MB, nbase, lane);
+#pragma unroll
+  for (int mt = 0; mt < MT; ++mt) {
+    const int rl0 = 16 * mt + g, r0 = t0 + rl0, r1 = r0 + 8;
+    if (DH_F32) {
+      // fp32 dh (the gradient feeding a LayerNorm backward), written from registers
+      float* dh = reinterpret_cast<float*>(p.dh);
+#pragma unroll
+      for (int nt = 0; nt < 8; ++nt) {
+        const int c = nbase + nt * 8 + 2 * t;
+        const float* x = v[mt][nt];
+        if (r0 < p.T) {
+          const float2 q0 = *reinterpret_cast<const float2*>(p.g + (size_t)r0 * H + c);
+          *reinterpret_cast<float2*>(dh + (size_t)r0 * H + c) = make_float2(x[0] + q0.x, x[1] + q0.y);
+        }
+        if (r1 < p.T) {
+          const float2 q1 = *reinterpret_cast<const float2*>(p.g + (size_t)r1 * H + c);
+          *reinterpret_cast<float2*>(dh + (size_t)r1 * H + c) = make_float2(x[2] + q1.x, x[3] + q1.y);
+        }
+      }
+      continue;
+    }
+    // dh goes through this warp's columns of the staged g rows, then out in whole row segments
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) {
       const int c = nbase + nt * 8 + 2 * t;
-      if (r0 < p.T) {
-        const float2 q0 = *reinterpret_cast<const float2*>(p.g + (size_t)r0 * H + c);
-        *reinterpret_cast<float2*>(dh + (size_t)r0 * H + c) = make_float2(v[nt][0] + q0.x, v[nt][1] + q0.y);
-      }
-      if (r1 < p.T) {
-        const float2 q1 = *reinterpret_cast<const float2*>(p.g + (size_t)r1 * H + c);
-        *reinterpret_cast<float2*>(dh + (size_t)r1 * H + c) = make_float2(v[nt][2] + q1.x, v[nt][3] + q1.y);
-      }
+      const float* x = v[mt][nt];
+      float2 q0 = make_float2(0.f, 0.f), q1 = make_float2(0.f, 0.f);
+      if (r0 < p.T) q0 = *reinterpret_cast<const float2*>(p.g + (size_t)r0 * H + c);
+      if (r1 < p.T) q1 = *reinterpret_cast<const float2*>(p.g + (size_t)r1 * H + c);
+      *reinterpret_cast<uint32_t*>(Gs + (size_t)rl0 * ldg + c) = pack2(x[0] + q0.x, x[1] + q0.y);
+      *reinterpret_cast<uint32_t*>(Gs + (size_t)(rl0 + 8) * ldg + c) = pack2(x[2] + q1.x, x[3] + q1.y);
     }
-    return;
+    __syncwarp();
+    store_block(reinterpret_cast<bf16*>(p.dh), H, Gs + 16 * mt * ldg, ldg, t0 + 16 * mt, p.T, nbase, lane);
   }
-  // dh goes through this warp's columns of the staged g rows, then out in whole row segments
-#pragma unroll
-  for (int nt = 0; nt < 8; ++nt) {
-    const int c = nbase + nt * 8 + 2 * t;
-    float2 q0 = make_float2(0.f, 0.f), q1 = make_float2(0.f, 0.f);
-    if (r0 < p.T) q0 = *reinterpret_cast<const float2*>(p.g + (size_t)r0 * H + c);
-    if (r1 < p.T) q1 = *reinterpret_cast<const float2*>(p.g + (size_t)r1 * H + c);
-    *reinterpret_cast<uint32_t*>(Gs + (size_t)g * ldg + c) = pack2(v[nt][0] + q0.x, v[nt][1] + q0.y);
-    *reinterpret_cast<uint32_t*>(Gs + (size_t)(g + 8) * ldg + c) = pack2(v[nt][2] + q1.x, v[nt][3] + q1.y);
-  }
-  __syncwarp();
-  store_block(reinterpret_cast<bf16*>(p.dh), H, Gs, ldg, t0, p.T, nbase, lane);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -709,10 +759,13 @@ __global__ void __launch_bounds__(256) adapter_dw_mma_kernel(DwArgs p) {
 }
 
 // shared memory of the backward row kernel
-size_t rows_smem(int H, int m) {
-  const int W = H / COLS_PER_WARP, W1 = H / phase1_slice(H, m);
+size_t rows_smem(int H, int m, int R) {
+  const int W = H / COLS_PER_WARP, W1 = H / phase1_slice(H, m, R);
   return (size_t)R * (H + 8) * 2 + (size_t)W1 * R * (m + 8) * 4 + (size_t)R * (m + 8) * 2 + (W * 16 + 16) * 4;
 }
+
+// 32 rows a CTA where that still gives every SM a tile (see RA_ROWS_BOUNDS)
+bool two_tiles(int T, int H) { return H <= 1024 && (T + 15) / 16 > device_sm_count(); }
 
 int smem_per_sm() {
   static int v = -1;
@@ -730,18 +783,20 @@ int smem_per_sm() {
 template <int MB, int MODE>
 cudaError_t launch_fwd(FwdArgs p, cudaStream_t st) {
   constexpr bool DEC = MODE == FWD_RMS;
+  const int R = two_tiles(p.T, p.H) ? 32 : 16;
   // gamma (and beta) go to shared memory when that keeps the CTAs per SM (1 KB reserved each)
   const int gbf = MODE == FWD_NONE ? 0 : (DEC ? 1 : 2) * p.H;
-  const size_t s0 = fwd_layout(p.H, MB, 0).bytes, s1 = fwd_layout(p.H, MB, gbf).bytes;
+  const size_t s0 = fwd_layout(p.H, MB, 0, R).bytes, s1 = fwd_layout(p.H, MB, gbf, R).bytes;
   const int per_sm = smem_per_sm();
   const bool aligned = MODE != FWD_NONE && ((uintptr_t)p.gamma & 15) == 0 &&
                        (DEC || ((uintptr_t)p.beta & 15) == 0);
-  p.stage_gb = aligned && s1 <= 220 * 1024 && per_sm > 0 &&
+  p.stage_gb = aligned && s1 <= 226 * 1024 && per_sm > 0 &&
                per_sm / (int)(s1 + 1024) == per_sm / (int)(s0 + 1024);
   const size_t smem = p.stage_gb ? s1 : s0;
   const int sz = size_class(p.H);
-  auto k = sz == 0 ? adapter_fwd_mma_kernel<MB, MODE, 0>
-         : sz == 1 ? adapter_fwd_mma_kernel<MB, MODE, 1> : adapter_fwd_mma_kernel<MB, MODE, 2>;
+  auto k = R == 32 ? (sz == 0 ? adapter_fwd_mma_kernel<MB, MODE, 0, 2> : adapter_fwd_mma_kernel<MB, MODE, 1, 2>)
+         : sz == 0 ? adapter_fwd_mma_kernel<MB, MODE, 0, 1>
+         : sz == 1 ? adapter_fwd_mma_kernel<MB, MODE, 1, 1> : adapter_fwd_mma_kernel<MB, MODE, 2, 1>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   e = launch_pdl(k, dim3((p.T + R - 1) / R), dim3((p.H / COLS_PER_WARP) * 32), smem, st, p);
@@ -751,10 +806,12 @@ cudaError_t launch_fwd(FwdArgs p, cudaStream_t st) {
 
 template <int MB, bool DH_F32>
 cudaError_t launch_bwd(const BwdArgs& p, cudaStream_t st) {
-  const size_t smem = rows_smem(p.H, MB);
+  const int R = two_tiles(p.T, p.H) ? 32 : 16;
+  const size_t smem = rows_smem(p.H, MB, R);
   const int sz = size_class(p.H);
-  auto k = sz == 0 ? adapter_bwd_rows_mma_kernel<MB, 0, DH_F32>
-         : sz == 1 ? adapter_bwd_rows_mma_kernel<MB, 1, DH_F32> : adapter_bwd_rows_mma_kernel<MB, 2, DH_F32>;
+  auto k = R == 32 ? (sz == 0 ? adapter_bwd_rows_mma_kernel<MB, 0, DH_F32, 2> : adapter_bwd_rows_mma_kernel<MB, 1, DH_F32, 2>)
+         : sz == 0 ? adapter_bwd_rows_mma_kernel<MB, 0, DH_F32, 1>
+         : sz == 1 ? adapter_bwd_rows_mma_kernel<MB, 1, DH_F32, 1> : adapter_bwd_rows_mma_kernel<MB, 2, DH_F32, 1>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   e = launch_pdl(k, dim3((p.T + R - 1) / R), dim3((p.H / COLS_PER_WARP) * 32), smem, st, p);
@@ -766,7 +823,7 @@ cudaError_t launch_bwd(const BwdArgs& p, cudaStream_t st) {
 
 bool adapter_mma_ok(int H, int m) {
   return H % 128 == 0 && H <= 2048 && (m == 32 || m == 64 || m == 128) &&
-         rows_smem(H, m) <= 220 * 1024 && fwd_layout(H, m, 0).bytes <= 220 * 1024;
+         rows_smem(H, m, 16) <= 220 * 1024 && fwd_layout(H, m, 0, 16).bytes <= 220 * 1024;
 }
 
 cudaError_t adapter_fwd_mma(const AdapterFwdArgs& a, const void* WdT_b, const void* WuT_b,
