@@ -1064,6 +1064,11 @@ bool tma_map_bf16(CUtensorMap* out, const void* ptr, int64_t rows, int64_t cols,
   return make_map(out, ptr, rows, cols, ld, box_cols, box_rows, DT_BF16);
 }
 
+bool tma_map_f32(CUtensorMap* out, const void* ptr, int64_t rows, int64_t cols, int64_t ld, int box_cols,
+                 int box_rows) {
+  return make_map(out, ptr, rows, cols, ld, box_cols, box_rows, DT_F32);
+}
+
 size_t gemm_sk_slot_bytes() { return (size_t)SK_SLOT_FLOATS * 4; }
 int gemm_sk_flags_per_slot() { return SK_MAX_WARPS; }
 

@@ -100,6 +100,9 @@ int device_sm_count();
 // 128-byte swizzle the tcgen05 operand descriptors read); false if the driver refuses it.
 bool tma_map_bf16(CUtensorMap* out, const void* ptr, int64_t rows, int64_t cols, int64_t ld, int box_cols,
                   int box_rows);
+// the same for float32
+bool tma_map_f32(CUtensorMap* out, const void* ptr, int64_t rows, int64_t cols, int64_t ld, int box_cols,
+                 int box_rows);
 
 // ---------------------------------------------------------------------------------------
 // Attention (per (batch, head); token t = b*S + s; head hh at columns hh*dh of q/k/v).
