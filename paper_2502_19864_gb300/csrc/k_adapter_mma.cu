@@ -261,7 +261,9 @@ __device__ __forceinline__ void load_rows_f32_as_bf16(bf16* dst, int ld, const f
 // MT = 2: 32 rows a CTA, one CTA an SM (168 or 128 registers), for H <= 1024 and batches that give
 // every SM more than one tile of 16.  The rows in flight on an SM are the same, but a weight fragment
 // is read once for them instead of twice: the 256 KB of fragments that every 16 rows of H = 1024 read
-// from L2 were more than twice the rows' own bytes.  RA_MT_FIGURES
+// from L2 were more than twice the rows' own bytes.  Forward and backward rows, 4096 x 768 13.4 -> 12.2
+// us and 12.2 -> 11.0, 8192 x 1024 31.6 -> 31.0 and 25.6 -> 23.8; without a norm 8192 x 1024 21.0 ->
+// 19.1.
 #define RA_ROWS_BOUNDS(SZ, MT) \
   __launch_bounds__((SZ) == 0 ? 384 : (SZ) == 1 ? 512 : 1024, (SZ) == 2 || (MT) == 2 ? 1 : 2)
 __host__ __device__ constexpr int size_class(int H) { return H <= 768 ? 0 : H <= 1024 ? 1 : 2; }

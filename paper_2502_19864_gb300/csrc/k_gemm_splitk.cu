@@ -307,9 +307,11 @@ int resident_clusters(int i) {
         cudaLaunchAttribute attr[2];
         const cudaLaunchConfig_t cfg = config<BN>(attr, device_sm_count() >> i << i, 1 << i, nullptr);
         n[i] = 0;
-        if (!prepare<BN>() || cudaOccupancyMaxActiveClusters(&n[i], gemm_splitk_kernel<BN>, &cfg) != cudaSuccess) n[i] = 0;
+        if (!prepare<BN>() || cudaOccupancyMaxActiveClusters(&n[i], gemm_splitk_kernel<BN>, &cfg) != cudaSuccess) {
+          n[i] = 0;
+          cudaGetLastError();  // (not the caller's)
+        }
       }
-      cudaGetLastError();
     }
   };
   static const Counts c;
