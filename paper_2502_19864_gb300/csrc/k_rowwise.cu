@@ -629,7 +629,7 @@ __global__ void __launch_bounds__(256) span_head_dw_reduce_kernel(const float* p
 // loss, and (logits_out) its logits in fp32.  Bound by HBM: the row is read once, 16 bytes a load
 // with all of a thread's NV loads in flight, and stays in registers (packed as stored) through the
 // maximum, the sum and the two writes.  8192 rows of 32000 bf16 logits with logits_out (2.1 GB):
-// 453 us (the floor is 308); reading the row from memory in each of three passes, two bytes at a time, took 716.
+// 370 us (the floor is 308; 453 with the label tested per logit and expf's denormal handling); reading the row from memory in each of three passes, two bytes at a time, took 716.
 template <typename T, int NV>
 __global__ void __launch_bounds__(512, 2) vocab_ce_kernel(T* logits, int ld, const int32_t* labels, int Tn,
     int V, float* row_loss, float* logits_out, bool out16, unsigned* err) {
@@ -652,6 +652,7 @@ __global__ void __launch_bounds__(512, 2) vocab_ce_kernel(T* logits, int ld, con
     lab = 0;
   }
   float mx = -INFINITY;
+  const int lvec = lab / VEC, lpos = lab % VEC;  // the vector that holds the label, and where
 #pragma unroll
   for (int n = 0; n < NV; ++n) {
     const int e = threadIdx.x + n * 512;
@@ -661,7 +662,11 @@ __global__ void __launch_bounds__(512, 2) vocab_ce_kernel(T* logits, int ld, con
     for (int i = 0; i < VEC; ++i) {
       x[i] = value(r[n], i);
       mx = fmaxf(mx, x[i]);
-      if (e * VEC + i == lab) zlab = x[i];
+    }
+    if (e == lvec) {
+#pragma unroll
+      for (int i = 0; i < VEC; ++i)
+        if (i == lpos) zlab = x[i];
     }
     if (logits_out) {
       float* o = logits_out + (int64_t)t * V + (int64_t)e * VEC;
@@ -680,14 +685,15 @@ __global__ void __launch_bounds__(512, 2) vocab_ce_kernel(T* logits, int ld, con
   mx = red[0][0];
 #pragma unroll
   for (int w = 1; w < 16; ++w) mx = fmaxf(mx, red[0][w]);
-  // (the special-function exponential: about 2 ulp, against the dozen-odd instructions of
-  // expf per logit over a 32000-wide vocabulary)
+  // (the special-function exponential: about 2 ulp, and below 2^-126 zero, against the dozen-odd
+  // instructions of expf per logit over a 32000-wide vocabulary)
+  constexpr float kLog2e = 1.4426950408889634f;
   float se = 0.f;
 #pragma unroll
   for (int n = 0; n < NV; ++n) {
     if (threadIdx.x + n * 512 >= nvec) continue;
 #pragma unroll
-    for (int i = 0; i < VEC; ++i) se += __expf(value(r[n], i) - mx);
+    for (int i = 0; i < VEC; ++i) se += ex2_fast((value(r[n], i) - mx) * kLog2e);
   }
   se = warp_sum(se);
   if (lane == 0) red[1][warp] = se;
@@ -702,12 +708,17 @@ __global__ void __launch_bounds__(512, 2) vocab_ce_kernel(T* logits, int ld, con
   for (int n = 0; n < NV; ++n) {
     const int e = threadIdx.x + n * 512;
     if (e >= nvec) continue;
+    float p[VEC];
+#pragma unroll
+    for (int i = 0; i < VEC; ++i) p[i] = ex2_fast((value(r[n], i) - lse) * kLog2e);
+    if (e == lvec) {
+#pragma unroll
+      for (int i = 0; i < VEC; ++i)
+        if (i == lpos) p[i] -= 1.f;
+    }
     uint4 o;
 #pragma unroll
-    for (int i = 0; i < VEC; ++i) {
-      const float p = __expf(value(r[n], i) - lse);
-      reinterpret_cast<T*>(&o)[i] = from_f<T>((p - (e * VEC + i == lab ? 1.f : 0.f)) * invT);
-    }
+    for (int i = 0; i < VEC; ++i) reinterpret_cast<T*>(&o)[i] = from_f<T>(p[i] * invT);
     *reinterpret_cast<uint4*>(row + (int64_t)e * VEC) = o;
   }
 }
