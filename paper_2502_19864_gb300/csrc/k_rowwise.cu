@@ -179,36 +179,68 @@ template <> __device__ __forceinline__ void st4<bf16>(void* p, int64_t i, float4
   *reinterpret_cast<uint2*>(reinterpret_cast<bf16*>(p) + i) = u;
 }
 
+// The norm backward kernels hold two arrays of the row.  At H = 2048 four warps share a row (each every
+// fourth 128 columns): with one, 182 registers left eight warps an SM, in step, and half the HBM rate
+// (RMSNorm, 8192 x 2048, 268 MB: 76.5 us; two warps 55; four 41.4, the floor is 39).  At 1024 two warps
+// a row changed nothing.
+constexpr int row_warps(int V) { return V >= 16 ? 4 : 1; }
+
+// (a, b) summed over the row's WPR warps, in warp order; every thread of the CTA calls it
+template <int WPR>
+__device__ __forceinline__ float2 row_sum2(float a, float b) {
+  a = warp_sum(a);
+  b = warp_sum(b);
+  if (WPR == 1) return make_float2(a, b);
+  __shared__ float2 red[8];
+  const int warp = threadIdx.x >> 5;
+  if ((threadIdx.x & 31) == 0) red[warp] = make_float2(a, b);
+  __syncthreads();
+  float2 s = red[warp / WPR * WPR];
+#pragma unroll
+  for (int w = 1; w < WPR; ++w) {
+    const float2 t = red[warp / WPR * WPR + w];
+    s.x += t.x;
+    s.y += t.y;
+  }
+  return s;
+}
+
 template <typename TX, int V>
 __global__ void __launch_bounds__(256) layernorm_bwd_vec_kernel(const float* dy, const float* dy2,
     const void* xhat, const float* rstd, const float* gamma, float* ds, void* ds_act, int Tn, int H) {
   pdl_wait();
   pdl_trigger();
-  const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (row >= Tn) return;
+  constexpr int WPR = row_warps(V), VL = V / WPR;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, row = blockIdx.x * (8 / WPR) + warp / WPR;
+  const bool live = row < Tn;
   const int64_t base = (int64_t)row * H;
-  float4 g[V], x[V];
+  auto col = [&](int v) { return ((v * WPR + warp % WPR) * 32 + lane) * 4; };
+  float4 g[VL], x[VL];
   float s1 = 0.f, s2 = 0.f;
+  if (live) {
 #pragma unroll
-  for (int v = 0; v < V; ++v) {
-    const int c = (v * 32 + lane) * 4;
-    float4 d = ld4<float>(dy, base + c);
-    if (dy2) {
-      const float4 d2 = ld4<float>(dy2, base + c);
-      d = make_float4(d.x + d2.x, d.y + d2.y, d.z + d2.z, d.w + d2.w);
+    for (int v = 0; v < VL; ++v) {
+      const int c = col(v);
+      float4 d = ld4<float>(dy, base + c);
+      if (dy2) {
+        const float4 d2 = ld4<float>(dy2, base + c);
+        d = make_float4(d.x + d2.x, d.y + d2.y, d.z + d2.z, d.w + d2.w);
+      }
+      const float4 gm = ld4<float>(gamma, c);
+      g[v] = make_float4(d.x * gm.x, d.y * gm.y, d.z * gm.z, d.w * gm.w);
+      x[v] = ld4<TX>(xhat, base + c);
+      s1 += g[v].x + g[v].y + g[v].z + g[v].w;
+      s2 += g[v].x * x[v].x + g[v].y * x[v].y + g[v].z * x[v].z + g[v].w * x[v].w;
     }
-    const float4 gm = ld4<float>(gamma, c);
-    g[v] = make_float4(d.x * gm.x, d.y * gm.y, d.z * gm.z, d.w * gm.w);
-    x[v] = ld4<TX>(xhat, base + c);
-    s1 += g[v].x + g[v].y + g[v].z + g[v].w;
-    s2 += g[v].x * x[v].x + g[v].y * x[v].y + g[v].z * x[v].z + g[v].w * x[v].w;
   }
-  s1 = warp_sum(s1) / H;
-  s2 = warp_sum(s2) / H;
+  const float2 s = row_sum2<WPR>(s1, s2);
+  if (!live) return;
+  s1 = s.x / H;
+  s2 = s.y / H;
   const float r = rstd[row];
 #pragma unroll
-  for (int v = 0; v < V; ++v) {
-    const int c = (v * 32 + lane) * 4;
+  for (int v = 0; v < VL; ++v) {
+    const int c = col(v);
     const float4 d = make_float4(r * (g[v].x - s1 - x[v].x * s2), r * (g[v].y - s1 - x[v].y * s2),
                                  r * (g[v].z - s1 - x[v].z * s2), r * (g[v].w - s1 - x[v].w * s2));
     st4<float>(ds, base + c, d);
@@ -286,24 +318,29 @@ __global__ void __launch_bounds__(256) rmsnorm_bwd_vec_kernel(const float* dy, c
     const float* gamma, const float* resid, float* dx, int Tn, int H) {
   pdl_wait();
   pdl_trigger();
-  const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if (row >= Tn) return;
+  constexpr int WPR = row_warps(V), VL = V / WPR;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, row = blockIdx.x * (8 / WPR) + warp / WPR;
+  const bool live = row < Tn;
   const int64_t base = (int64_t)row * H;
-  float4 g[V], a[V];
+  auto col = [&](int v) { return ((v * WPR + warp % WPR) * 32 + lane) * 4; };
+  float4 g[VL], a[VL];
   float s = 0.f;
+  if (live) {
 #pragma unroll
-  for (int v = 0; v < V; ++v) {
-    const int c = (v * 32 + lane) * 4;
-    const float4 d = ld4<float>(dy, base + c), gm = ld4<float>(gamma, c);
-    g[v] = make_float4(d.x * gm.x, d.y * gm.y, d.z * gm.z, d.w * gm.w);
-    a[v] = ld4<float>(x, base + c);
-    s += g[v].x * a[v].x + g[v].y * a[v].y + g[v].z * a[v].z + g[v].w * a[v].w;
+    for (int v = 0; v < VL; ++v) {
+      const int c = col(v);
+      const float4 d = ld4<float>(dy, base + c), gm = ld4<float>(gamma, c);
+      g[v] = make_float4(d.x * gm.x, d.y * gm.y, d.z * gm.z, d.w * gm.w);
+      a[v] = ld4<float>(x, base + c);
+      s += g[v].x * a[v].x + g[v].y * a[v].y + g[v].z * a[v].z + g[v].w * a[v].w;
+    }
   }
-  s = warp_sum(s) / H;
+  s = row_sum2<WPR>(s, 0.f).x / H;
+  if (!live) return;
   const float r = rstd[row], k = r * r * r * s;
 #pragma unroll
-  for (int v = 0; v < V; ++v) {
-    const int c = (v * 32 + lane) * 4;
+  for (int v = 0; v < VL; ++v) {
+    const int c = col(v);
     const float4 q = resid ? ld4<float>(resid, base + c) : make_float4(0.f, 0.f, 0.f, 0.f);
     st4<float>(dx, base + c, make_float4(q.x + r * g[v].x - a[v].x * k, q.y + r * g[v].y - a[v].y * k,
                                          q.z + r * g[v].z - a[v].z * k, q.w + r * g[v].w - a[v].w * k));
@@ -1031,6 +1068,7 @@ cudaError_t layernorm_bwd(const float* dy, const float* dy2, const void* xhat, c
                           cudaStream_t st, void* ds_act) {
   unsigned grid = blocks_for((int64_t)T * 32, 256);
   if (const int V = row_vec(H)) {
+    grid = blocks_for((int64_t)T * 32 * row_warps(V), 256);
     if (dtype == DT_BF16) RA_VEC_SWITCH(V, ((void)launch_pdl(layernorm_bwd_vec_kernel<bf16, VV>, dim3(grid), dim3(256), (size_t)0, st, dy, dy2, xhat, rstd, gamma, ds, ds_act, T, H)))
     else RA_VEC_SWITCH(V, ((void)launch_pdl(layernorm_bwd_vec_kernel<float, VV>, dim3(grid), dim3(256), (size_t)0, st, dy, dy2, xhat, rstd, gamma, ds, ds_act, T, H)))
   } else if (dtype == DT_BF16) {
@@ -1089,7 +1127,7 @@ cudaError_t rmsnorm_fwd(const void* x, int x_dtype, const float* gamma, float ep
 cudaError_t rmsnorm_bwd(const float* dy, const float* x, const float* rstd, const float* gamma,
                         const float* resid, float* dx, int T, int H, cudaStream_t st) {
   if (const int V = row_vec(H))
-    RA_VEC_SWITCH(V, ((void)launch_pdl(rmsnorm_bwd_vec_kernel<VV>, dim3(blocks_for((int64_t)T * 32, 256)), dim3(256), (size_t)0, st, dy, x, rstd, gamma, resid, dx, T, H)))
+    RA_VEC_SWITCH(V, ((void)launch_pdl(rmsnorm_bwd_vec_kernel<VV>, dim3(blocks_for((int64_t)T * 32 * row_warps(VV), 256)), dim3(256), (size_t)0, st, dy, x, rstd, gamma, resid, dx, T, H)))
   else
     (void)launch_pdl(rmsnorm_bwd_kernel, dim3(blocks_for((int64_t)T * 32, 256)), dim3(256), (size_t)0, st, dy, x, rstd, gamma, resid, dx, T, H);
   note_launch(1);
