@@ -42,10 +42,6 @@ constexpr float kLog2e = 1.4426950408889634f;
 constexpr int BR = 128;          // rows of a query or key block
 constexpr int NTHR = 256;        // 8 warps
 
-__device__ __forceinline__ void cp_async16b(uint32_t dst, const void* src, bool valid) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(valid ? 16 : 0)
-               : "memory");
-}
 __device__ __forceinline__ uint32_t pk2(float a, float b) {
   __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<uint32_t*>(&h);
@@ -68,20 +64,8 @@ struct BwdPlan {
   static constexpr uint32_t TMEM_COLS = 128 + 2 * DH <= 256 ? 256 : 512;
 };
 
-// cp.async copies of rows [r0, r0 + 128) of one head's DH columns (base points at the head's
-// first column of row 0; row stride ld elements) into a swizzled 128 x DH block; rows at or
-// beyond S are zero-filled
-template <int DH>
-__device__ __forceinline__ void load_block(uint32_t dst, const bf16* base, int ld, int r0, int S) {
-  constexpr int CH = DH / 8;  // 16-byte chunks per row
-  for (int e = threadIdx.x; e < BR * CH; e += NTHR) {
-    const int r = e / CH, j = e % CH, g = r0 + r;
-    const bool ok = g < S;
-    cp_async16b(dst + (j >> 3) * (BR * 128) + swz(r, j & 7), base + (size_t)(ok ? g : 0) * ld + 8 * j, ok);
-  }
-}
-// the same block by TMA: rows [row, row + 128) of a [tokens, columns] matrix from column col on, one
-// box per 64-wide atom.  Rows at or beyond S hold the next sequence's (zeros past the last token):
+// Rows [row, row + 128) of a [tokens, columns] matrix, columns from col on, into a swizzled 128 x DH
+// block by TMA, one box per 64-wide atom.  Rows at or beyond S hold the next sequence's (zeros past the last token):
 // their probabilities are zero.
 template <int DH>
 __device__ __forceinline__ void tma_block(const CUtensorMap* tm, uint32_t dst, uint64_t* bar, int col, int row) {
@@ -569,10 +553,11 @@ struct FwdPlan {
 // blockIdx.x counts query blocks from the last: with a causal mask the blocks with the most
 // key blocks start first
 template <int DH, bool CAUSAL>
-__global__ void __launch_bounds__(NTHR, 2) attn_fwd_blocks_tc_kernel(AttnArgs a) {
+__global__ void __launch_bounds__(NTHR, 2) attn_fwd_blocks_tc_kernel(
+    const __grid_constant__ CUtensorMap tmQKV, AttnArgs a) {
   using Pl = FwdPlan<DH>;
   extern __shared__ __align__(1024) uint8_t smem[];
-  __shared__ __align__(8) uint64_t bar;
+  __shared__ __align__(8) uint64_t bar, q_bar, kv_bar[2];
   __shared__ uint32_t tmem_sh;
   __shared__ volatile int abort_sh;
   const uint32_t sb = smem_u32(smem);
@@ -584,15 +569,30 @@ __global__ void __launch_bounds__(NTHR, 2) attn_fwd_blocks_tc_kernel(AttnArgs a)
   const int quad = warp & 3, half = warp >> 2;
   const int S = a.S, NB = (S + BR - 1) / BR;
   const int i = NB - 1 - (int)blockIdx.x, bh = blockIdx.y, b = bh / a.n_heads, hh = bh % a.n_heads;
-  const int H = a.n_heads * DH, ld = 3 * H;
-  const bf16* qkv = reinterpret_cast<const bf16*>(a.qkv) + (size_t)b * S * ld + hh * DH;
+  const int H = a.n_heads * DH;
   float (*red)[2][BR] = reinterpret_cast<float (*)[2][BR]>(smem + Pl::RED);  // [m | l][half][row]
   const float sl2 = a.scale * kLog2e;
 
-  if (tid == 0) {
-    mbar_init(&bar, 1);
-    abort_sh = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  // q, k or v (part 0, 1, 2) rows of block blk_ into a block of shared memory; one lane calls it
+  auto load = [&](uint32_t dst, uint64_t* lb, int part, int blk_) {
+    mbar_expect_tx(lb, BR * DH * 2);
+    tma_block<DH>(&tmQKV, dst, lb, part * H + hh * DH, b * S + blk_ * BR);
+  };
+  if (warp == 1) {
+    // this warp starts the first copies while warp 0 allocates TMEM
+    if (elect_one()) {
+      mbar_init(&bar, 1);
+      mbar_init(&q_bar, 1);
+      mbar_init(&kv_bar[0], 1);
+      mbar_init(&kv_bar[1], 1);
+      abort_sh = 0;
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      pdl_wait();
+      load(sb + Pl::Q, &q_bar, 0, i);
+      load(sb + Pl::K, &kv_bar[0], 1, 0);
+    }
+    __syncwarp();
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_sh)),
@@ -614,8 +614,7 @@ __global__ void __launch_bounds__(NTHR, 2) attn_fwd_blocks_tc_kernel(AttnArgs a)
   bool pending = false;
   bool ok = true;
   auto wait_mma = [&]() {
-    if (ok) {
-      mbar_wait(&bar, phase, &abort_sh, a.err);
+    if (ok && mbar_wait(&bar, phase, &abort_sh, a.err)) {
       phase ^= 1u;
       pending = false;
     }
@@ -630,23 +629,35 @@ __global__ void __launch_bounds__(NTHR, 2) attn_fwd_blocks_tc_kernel(AttnArgs a)
     __syncthreads();
     tc_fence_after();
   };
-  auto copies_done = [&]() {
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
+  // every thread waits for the copies into buffer x; then a barrier as above
+  uint32_t kv_phase = 0u, loading = 1u;  // a bit per buffer: its phase; copies not yet waited for
+  auto copied = [&](int x) {
+    if (ok && mbar_wait(&kv_bar[x], (kv_phase >> x) & 1u, &abort_sh, a.err)) {
+      kv_phase ^= 1u << x;
+      loading &= ~(1u << x);
+    }
+    publish();
+    ok = ok && abort_sh == 0;
   };
   auto live = [&](int key) { return q < S && key < S && (!CAUSAL || key <= q); };
   constexpr uint32_t ID128 = idesc_bf16(BR, BR);
   const int j_end = CAUSAL ? i + 1 : NB;
 
-  load_block<DH>(sb + Pl::Q, qkv, ld, i * BR, S);
-  // ---- pass 1: the row's max and sum of exp (log2 units of the scaled scores)
+  bool q_loading = true;
+  if (mbar_wait(&q_bar, 0, &abort_sh, a.err)) q_loading = false;
+  // ---- pass 1: the row's max and sum of exp (log2 units of the scaled scores); the key blocks take
+  // turns in the spaces of k and v, the next one on its way while one is used
   float m = -INFINITY, l = 0.f;
   for (int j = 0; j < j_end && ok; ++j) {
-    load_block<DH>(sb + Pl::K, qkv + H, ld, j * BR, S);
-    copies_done();
-    publish();
+    const int x = j & 1;
+    if (j + 1 < j_end) {
+      if (warp == 1 && elect_one()) load(sb + (x ? Pl::K : Pl::V), &kv_bar[x ^ 1], 1, j + 1);
+      loading |= 2u >> x;
+    }
+    copied(x);
+    if (!ok) break;
     if (warp == 0 && elect_one()) {
-      mma_qk<DH>(tmem + Pl::C_S, sb + Pl::Q, sb + Pl::K, ID128);
+      mma_qk<DH>(tmem + Pl::C_S, sb + Pl::Q, sb + (x ? Pl::V : Pl::K), ID128);
       umma_commit(&bar);
     }
     pending = true;
@@ -691,12 +702,13 @@ __global__ void __launch_bounds__(NTHR, 2) attn_fwd_blocks_tc_kernel(AttnArgs a)
   const float lse2 = M > -INFINITY ? M + log2f(L) : 0.f;
   // ---- pass 2: P = exp(scale S - lse), O += P v_j
   for (int j = 0; j < j_end && ok; ++j) {
-    load_block<DH>(sb + Pl::K, qkv + H, ld, j * BR, S);
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    load_block<DH>(sb + Pl::V, qkv + 2 * H, ld, j * BR, S);  // lands while S is computed
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    asm volatile("cp.async.wait_group 1;" ::: "memory");      // k_j
-    publish();
+    if (warp == 1 && elect_one()) {
+      load(sb + Pl::K, &kv_bar[0], 1, j);
+      load(sb + Pl::V, &kv_bar[1], 2, j);  // lands while S is computed
+    }
+    loading = 3u;
+    copied(0);  // k_j
+    if (!ok) break;
     if (warp == 0 && elect_one()) {
       mma_qk<DH>(tmem + Pl::C_S, sb + Pl::Q, sb + Pl::K, ID128);
       umma_commit(&bar);
@@ -726,8 +738,8 @@ __global__ void __launch_bounds__(NTHR, 2) attn_fwd_blocks_tc_kernel(AttnArgs a)
         *reinterpret_cast<uint4*>(xrow + swz(row, 4 * h2 + g)) = make_uint4(w[0], w[1], w[2], w[3]);
       }
     }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");  // v_j
-    publish();
+    copied(1);  // v_j (and P)
+    if (!ok) break;
     if (warp == 0 && elect_one()) {
       mma_xb<DH>(tmem + Pl::C_O, sb + Pl::X, sb + Pl::V, j > 0);
       umma_commit(&bar);
@@ -752,9 +764,14 @@ __global__ void __launch_bounds__(NTHR, 2) attn_fwd_blocks_tc_kernel(AttnArgs a)
     }
     if (a.lse && half == 0 && q < S) a.lse[(size_t)bh * S + q] = lse2 * 0.69314718055994531f;
   }
-  if (pending) {
+  if (pending || q_loading || loading) {
+    // a wait gave up: let the issued copies and products finish before shared memory and TMEM are
+    // released
     volatile int no_abort = 0;
-    mbar_wait(&bar, phase, &no_abort, nullptr);
+    if (pending) mbar_wait(&bar, phase, &no_abort, nullptr);
+    if (q_loading) mbar_wait(&q_bar, 0, &no_abort, nullptr);
+    for (int x = 0; x < 2; ++x)
+      if (loading >> x & 1u) mbar_wait(&kv_bar[x], (kv_phase >> x) & 1u, &no_abort, nullptr);
   }
   tc_fence_before();
   __syncthreads();
@@ -775,7 +792,10 @@ cudaError_t launch_fwd_blocks(const AttnArgs& a, cudaStream_t st) {
     attr = true;
   }
   const int nb = (a.S + BR - 1) / BR;
-  cudaError_t e = launch_pdl(k, dim3(nb, a.B * a.n_heads), dim3(NTHR), (size_t)FwdPlan<DH>::BYTES, st, a);  // x: reversed
+  CUtensorMap mq;  // qkv [B S, 3 H] in boxes of 64 columns x 128 rows
+  const int H = a.n_heads * DH;
+  if (!tma_map_bf16(&mq, a.qkv, (int64_t)a.B * a.S, 3LL * H, 3LL * H, 64, BR)) return cudaErrorNotSupported;
+  cudaError_t e = launch_pdl(k, dim3(nb, a.B * a.n_heads), dim3(NTHR), (size_t)FwdPlan<DH>::BYTES, st, mq, a);  // x: reversed
   note_launch(1);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -784,7 +804,7 @@ cudaError_t launch_fwd_blocks(const AttnArgs& a, cudaStream_t st) {
 
 bool attention_fwd_blocks_tc_ok(const AttnArgs& a) {
   return a.dtype == DT_BF16 && (a.head_dim == 64 || a.head_dim == 128) && a.S >= 1 &&
-         (!a.rope || a.qk_rotated);
+         (!a.rope || a.qk_rotated) && (reinterpret_cast<uintptr_t>(a.qkv) & 15) == 0;
 }
 
 cudaError_t attention_fwd_blocks_tc(const AttnArgs& a, cudaStream_t st) {

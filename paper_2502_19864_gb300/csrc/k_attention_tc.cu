@@ -76,13 +76,24 @@ __global__ void __launch_bounds__(256) attn_fwd_tc_kernel(const __grid_constant_
   const int H = a.n_heads * DH, S = a.S;
   const int q0 = blockIdx.x * QT;
 
-  if (tid == 0) {
-    mbar_init(&mma_bar, 1);
-    mbar_init(&load_bar, 1);
-    abort_sh = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmQ)) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmKV)) : "memory");
+  // q, k and v: one box each from the [B S, 3 H] qkv matrix (x = the head's columns), asked for by
+  // this warp while warp 0 allocates TMEM (about 1200 cycles)
+  if (warp == 1) {
+    if (elect_one()) {
+      mbar_init(&mma_bar, 1);
+      mbar_init(&load_bar, 1);
+      abort_sh = 0;
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmQ)) : "memory");
+      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmKV)) : "memory");
+      pdl_wait();
+      mbar_expect_tx(&load_bar, (uint32_t)(QT + 2 * NK) * 128);
+      tma_load_2d_at(&tmQ, sbase + Pl::Q_OFF, &load_bar, hh * DH, b * S + q0);
+      tma_load_2d_at(&tmKV, sbase + Pl::K_OFF, &load_bar, H + hh * DH, b * S);
+      tma_load_2d_at(&tmKV, sbase + Pl::V_OFF, &load_bar, 2 * H + hh * DH, b * S);
+    }
+    __syncwarp();
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -97,13 +108,6 @@ __global__ void __launch_bounds__(256) attn_fwd_tc_kernel(const __grid_constant_
   pdl_wait();
   pdl_trigger();
 
-  // q, k and v: one box each from the [B S, 3 H] qkv matrix (x = the head's columns)
-  if (warp == 0 && elect_one()) {
-    mbar_expect_tx(&load_bar, (uint32_t)(QT + 2 * NK) * 128);
-    tma_load_2d_at(&tmQ, sbase + Pl::Q_OFF, &load_bar, hh * DH, b * S + q0);
-    tma_load_2d_at(&tmKV, sbase + Pl::K_OFF, &load_bar, H + hh * DH, b * S);
-    tma_load_2d_at(&tmKV, sbase + Pl::V_OFF, &load_bar, 2 * H + hh * DH, b * S);
-  }
   bool ok = mbar_wait(&load_bar, 0, &abort_sh, a.err);
   tc_fence_after();
 
