@@ -64,17 +64,17 @@ struct BwdPlan {
   static constexpr uint32_t TMEM_COLS = 128 + 2 * DH <= 256 ? 256 : 512;
 };
 
-// Rows [row, row + 128) of a [tokens, columns] matrix, columns from col on, into a swizzled 128 x DH
-// block by TMA, one box per 64-wide atom.  Rows at or beyond S hold the next sequence's (zeros past the last token):
-// their probabilities are zero.
+// Rows [row, row + 128) of sequence b of a [B, S, columns] matrix, columns from col on, into a swizzled 128 x
+// DH block by TMA, one box per 64-wide atom.  Rows at or beyond S arrive as zeros: their probabilities are
+// zero, which times another sequence's values would not be zero where those are not finite.
 template <int DH>
-__device__ __forceinline__ void tma_block(const CUtensorMap* tm, uint32_t dst, uint64_t* bar, int col, int row) {
+__device__ __forceinline__ void tma_block(const CUtensorMap* tm, uint32_t dst, uint64_t* bar, int col, int row, int b) {
 #pragma unroll
   for (int n = 0; n < DH / 64; ++n)
     asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3}], [%4];" ::"r"(dst + n * (BR * 128)),
-        "l"(reinterpret_cast<uint64_t>(tm)), "r"(col + 64 * n), "r"(row), "r"(smem_u32(bar))
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst + n * (BR * 128)),
+        "l"(reinterpret_cast<uint64_t>(tm)), "r"(col + 64 * n), "r"(row), "r"(b), "r"(smem_u32(bar))
         : "memory");
 }
 // D[128 x 128] = A B^T over K = DH (both K-major 128 x DH blocks)
@@ -149,9 +149,9 @@ __global__ void __launch_bounds__(NTHR, DH == 64 ? 2 : 1) attn_bwd_tc_kernel(con
   constexpr uint32_t BLK_BYTES = BR * DH * 2;
   // q, k or v (part 0, 1, 2) rows of block blk_, or dO's, into a block of shared memory
   auto load_qkv = [&](uint32_t dst, int part, int blk_) {
-    tma_block<DH>(&tmQKV, dst, &load_bar, part * H + hh * DH, b * S + blk_ * BR);
+    tma_block<DH>(&tmQKV, dst, &load_bar, part * H + hh * DH, blk_ * BR, b);
   };
-  auto load_do = [&](uint32_t dst, int blk_) { tma_block<DH>(&tmDO, dst, &load_bar, hh * DH, b * S + blk_ * BR); };
+  auto load_do = [&](uint32_t dst, int blk_) { tma_block<DH>(&tmDO, dst, &load_bar, hh * DH, blk_ * BR, b); };
   if (warp == 1) {
     // this warp starts the first copies while warp 0 allocates TMEM (about 1200 cycles)
     if (elect_one()) {
@@ -509,11 +509,11 @@ cudaError_t launch_bwd_tc(const AttnArgs& a, cudaStream_t st) {
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = FUSED ? 2 : 1;
-  // qkv [B S, 3 H] and dO [B S, H] in boxes of 64 columns x 128 rows
+  // qkv [B, S, 3 H] and dO [B, S, H] in boxes of 64 columns x 128 rows of one sequence
   const int H = a.n_heads * DH;
   CUtensorMap mq, md;
-  if (!tma_map_bf16(&mq, a.qkv, (int64_t)a.B * a.S, 3LL * H, 3LL * H, 64, BR) ||
-      !tma_map_bf16(&md, a.dO, (int64_t)a.B * a.S, H, H, 64, BR))
+  if (!tma_map_bf16_batch(&mq, a.qkv, a.B, a.S, 3LL * H, 3LL * H, 64, BR) ||
+      !tma_map_bf16_batch(&md, a.dO, a.B, a.S, H, H, 64, BR))
     return cudaErrorNotSupported;
   cudaError_t e = cudaLaunchKernelEx(&cfg, k, mq, md, a);
   note_launch(1);
@@ -576,7 +576,7 @@ __global__ void __launch_bounds__(NTHR, 2) attn_fwd_blocks_tc_kernel(
   // q, k or v (part 0, 1, 2) rows of block blk_ into a block of shared memory; one lane calls it
   auto load = [&](uint32_t dst, uint64_t* lb, int part, int blk_) {
     mbar_expect_tx(lb, BR * DH * 2);
-    tma_block<DH>(&tmQKV, dst, lb, part * H + hh * DH, b * S + blk_ * BR);
+    tma_block<DH>(&tmQKV, dst, lb, part * H + hh * DH, blk_ * BR, b);
   };
   if (warp == 1) {
     // this warp starts the first copies while warp 0 allocates TMEM
@@ -792,9 +792,9 @@ cudaError_t launch_fwd_blocks(const AttnArgs& a, cudaStream_t st) {
     attr = true;
   }
   const int nb = (a.S + BR - 1) / BR;
-  CUtensorMap mq;  // qkv [B S, 3 H] in boxes of 64 columns x 128 rows
+  CUtensorMap mq;  // qkv [B, S, 3 H] in boxes of 64 columns x 128 rows of one sequence
   const int H = a.n_heads * DH;
-  if (!tma_map_bf16(&mq, a.qkv, (int64_t)a.B * a.S, 3LL * H, 3LL * H, 64, BR)) return cudaErrorNotSupported;
+  if (!tma_map_bf16_batch(&mq, a.qkv, a.B, a.S, 3LL * H, 3LL * H, 64, BR)) return cudaErrorNotSupported;
   cudaError_t e = launch_pdl(k, dim3(nb, a.B * a.n_heads), dim3(NTHR), (size_t)FwdPlan<DH>::BYTES, st, mq, a);  // x: reversed
   note_launch(1);
   return e != cudaSuccess ? e : cudaGetLastError();

@@ -944,17 +944,18 @@ EncodeTiledFn encode_fn() {
 struct MapKey {
   const void* ptr;
   int64_t rows, cols, ld;
-  int box_cols, box_rows, dtype, blocks;
+  int box_cols, box_rows, dtype, blocks, batch;
   bool operator==(const MapKey& o) const {
     return ptr == o.ptr && rows == o.rows && cols == o.cols && ld == o.ld &&
-           box_cols == o.box_cols && box_rows == o.box_rows && dtype == o.dtype && blocks == o.blocks;
+           box_cols == o.box_cols && box_rows == o.box_rows && dtype == o.dtype && blocks == o.blocks &&
+           batch == o.batch;
   }
 };
 struct MapKeyHash {
   size_t operator()(const MapKey& k) const {
     size_t h = std::hash<const void*>()(k.ptr);
     h ^= std::hash<int64_t>()(k.rows * 1000003 + k.cols) + 0x9e3779b9 + (h << 6) + (h >> 2);
-    h ^= std::hash<int64_t>()(k.ld * 31 + k.box_rows * 7 + k.box_cols * 131 + k.dtype + k.blocks * 1009) +
+    h ^= std::hash<int64_t>()(k.ld * 31 + k.box_rows * 7 + k.box_cols * 131 + k.dtype + k.blocks * 1009 + k.batch * 8191) +
          0x9e3779b9 + (h << 6) + (h >> 2);
     return h;
   }
@@ -968,11 +969,13 @@ struct MapKeyHash {
 // blocks > 0: the matrix (cols a multiple of box_cols) seen in 3-D as (box_cols columns, rows,
 // cols / box_cols column blocks); one box of box_cols x box_rows x blocks then lands as
 // `blocks` consecutive box_cols x box_rows tiles (the MN-major B operand atoms).
+// batch > 0: `batch` such matrices one after the other, as (cols, rows, batch); a box stays within
+// one of them, with zeros for its rows past the matrix's last.
 bool make_map(CUtensorMap* out, const void* ptr, int64_t rows, int64_t cols, int64_t ld,
-              int box_cols, int box_rows, int dtype, int blocks = 0) {
+              int box_cols, int box_rows, int dtype, int blocks = 0, int batch = 0) {
   static std::mutex mu;
   static std::unordered_map<MapKey, CUtensorMap, MapKeyHash> cache;
-  MapKey key{ptr, rows, cols, ld, box_cols, box_rows, dtype, blocks};
+  MapKey key{ptr, rows, cols, ld, box_cols, box_rows, dtype, blocks, batch};
   std::lock_guard<std::mutex> lock(mu);
   auto it = cache.find(key);
   if (it != cache.end()) {
@@ -988,12 +991,13 @@ bool make_map(CUtensorMap* out, const void* ptr, int64_t rows, int64_t cols, int
                                            : CU_TENSOR_MAP_SWIZZLE_NONE;
   const bool b3 = blocks > 0;
   if (b3 && cols % box_cols) return false;
-  cuuint64_t gdim[3] = {(cuuint64_t)(b3 ? box_cols : cols), (cuuint64_t)rows, (cuuint64_t)(b3 ? cols / box_cols : 1)};
-  cuuint64_t gstride[2] = {(cuuint64_t)ld * es, (cuuint64_t)box_cols * es};
+  cuuint64_t gdim[3] = {(cuuint64_t)(b3 ? box_cols : cols), (cuuint64_t)rows,
+                        (cuuint64_t)(b3 ? cols / box_cols : batch ? batch : 1)};
+  cuuint64_t gstride[2] = {(cuuint64_t)ld * es, (cuuint64_t)(batch ? rows * ld : box_cols) * es};
   cuuint32_t box[3] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows, (cuuint32_t)(b3 ? blocks : 1)};
   cuuint32_t estride[3] = {1, 1, 1};
   CUresult r = fn(out, dtype == DT_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
-                  b3 ? 3 : 2, const_cast<void*>(ptr), gdim, gstride, box, estride,
+                  b3 || batch ? 3 : 2, const_cast<void*>(ptr), gdim, gstride, box, estride,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return false;
@@ -1062,6 +1066,11 @@ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 
 bool tma_map_bf16(CUtensorMap* out, const void* ptr, int64_t rows, int64_t cols, int64_t ld, int box_cols,
                   int box_rows) {
   return make_map(out, ptr, rows, cols, ld, box_cols, box_rows, DT_BF16);
+}
+
+bool tma_map_bf16_batch(CUtensorMap* out, const void* ptr, int batch, int64_t rows, int64_t cols, int64_t ld,
+                        int box_cols, int box_rows) {
+  return make_map(out, ptr, rows, cols, ld, box_cols, box_rows, DT_BF16, 0, batch);
 }
 
 bool tma_map_f32(CUtensorMap* out, const void* ptr, int64_t rows, int64_t cols, int64_t ld, int box_cols,

@@ -100,7 +100,11 @@ int device_sm_count();
 // 128-byte swizzle the tcgen05 operand descriptors read); false if the driver refuses it.
 bool tma_map_bf16(CUtensorMap* out, const void* ptr, int64_t rows, int64_t cols, int64_t ld, int box_cols,
                   int box_rows);
-// the same for float32
+// 3-D tensor map (columns, rows, batch) of `batch` such matrices one after the other: a box's rows past
+// the last of its own matrix arrive as zeros, not as the next one's
+bool tma_map_bf16_batch(CUtensorMap* out, const void* ptr, int batch, int64_t rows, int64_t cols, int64_t ld,
+                        int box_cols, int box_rows);
+// the 2-D map for float32
 bool tma_map_f32(CUtensorMap* out, const void* ptr, int64_t rows, int64_t cols, int64_t ld, int box_cols,
                  int box_rows);
 
