@@ -12,9 +12,8 @@
 //     as stored, MN-major through the descriptor (no transposed copy); O / sum and the
 //     log-sum-exp (natural log of the scaled scores) go to memory.
 // p reuses the shared memory of q and k, so two CTAs fit per SM.  All keys fit in one tile,
-// so the softmax is exact in one pass (no running rescale).  Key rows at or beyond S hold
-// the next sequence's keys (or, past the last token, the copy's zero fill): they get p = 0,
-// and query rows beyond S are not stored.
+// so the softmax is exact in one pass (no running rescale).  Rows at or beyond S arrive as zeros
+// (a box stays within its sequence): their keys get p = 0, and query rows beyond S are not stored.
 #include "common.cuh"
 #include "kernels.h"
 #include "tcgen05.cuh"
@@ -47,11 +46,12 @@ struct AttnTcPlan {
   static constexpr uint32_t TMEM_COLS = NK;            // S; O reuses columns [0, 64)
 };
 
-__device__ __forceinline__ void tma_load_2d_at(const CUtensorMap* tm, uint32_t dst, uint64_t* bar, int c0, int c1) {
+__device__ __forceinline__ void tma_load_3d_at(const CUtensorMap* tm, uint32_t dst, uint64_t* bar, int c0, int c1,
+                                               int c2) {
   asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(tm)), "r"(c0), "r"(c1), "r"(smem_u32(bar))
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(tm)), "r"(c0), "r"(c1), "r"(c2), "r"(smem_u32(bar))
       : "memory");
 }
 
@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(256) attn_fwd_tc_kernel(const __grid_constant_
   const int H = a.n_heads * DH, S = a.S;
   const int q0 = blockIdx.x * QT;
 
-  // q, k and v: one box each from the [B S, 3 H] qkv matrix (x = the head's columns), asked for by
+  // q, k and v: one box each from the [B, S, 3 H] qkv matrix (x = the head's columns), asked for by
   // this warp while warp 0 allocates TMEM (about 1200 cycles)
   if (warp == 1) {
     if (elect_one()) {
@@ -89,9 +89,9 @@ __global__ void __launch_bounds__(256) attn_fwd_tc_kernel(const __grid_constant_
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmKV)) : "memory");
       pdl_wait();
       mbar_expect_tx(&load_bar, (uint32_t)(QT + 2 * NK) * 128);
-      tma_load_2d_at(&tmQ, sbase + Pl::Q_OFF, &load_bar, hh * DH, b * S + q0);
-      tma_load_2d_at(&tmKV, sbase + Pl::K_OFF, &load_bar, H + hh * DH, b * S);
-      tma_load_2d_at(&tmKV, sbase + Pl::V_OFF, &load_bar, 2 * H + hh * DH, b * S);
+      tma_load_3d_at(&tmQ, sbase + Pl::Q_OFF, &load_bar, hh * DH, q0, b);
+      tma_load_3d_at(&tmKV, sbase + Pl::K_OFF, &load_bar, H + hh * DH, 0, b);
+      tma_load_3d_at(&tmKV, sbase + Pl::V_OFF, &load_bar, 2 * H + hh * DH, 0, b);
     }
     __syncwarp();
   }
@@ -241,11 +241,11 @@ cudaError_t launch_tc(const AttnArgs& a, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     attr = true;
   }
-  // the qkv matrix [B S, 3 H]: q boxes of 64 columns x 128 rows, k and v boxes of NK rows
+  // the qkv matrix [B, S, 3 H]: q boxes of 64 columns x 128 rows, k and v boxes of NK rows
   const int H = a.n_heads * DH;
   CUtensorMap mq, mkv;
-  if (!tma_map_bf16(&mq, a.qkv, (int64_t)a.B * a.S, 3LL * H, 3LL * H, DH, QT) ||
-      !tma_map_bf16(&mkv, a.qkv, (int64_t)a.B * a.S, 3LL * H, 3LL * H, DH, NK))
+  if (!tma_map_bf16_batch(&mq, a.qkv, a.B, a.S, 3LL * H, 3LL * H, DH, QT) ||
+      !tma_map_bf16_batch(&mkv, a.qkv, a.B, a.S, 3LL * H, 3LL * H, DH, NK))
     return cudaErrorNotSupported;
   cudaError_t e = launch_pdl(k, dim3((a.S + QT - 1) / QT, a.B * a.n_heads), dim3(256),
                              (size_t)AttnTcPlan<NK>::SMEM, st, mq, mkv, a);

@@ -43,3 +43,8 @@ def check_apart(cfg):
     synth._enc(2, 128, 2, 256, 32, 2, 300, "bf16"), synth._enc(2, 256, 2, 256, 32, 2, 77, "bf16")], ids=str)
 def test_blocks_of_128(cfg):
     check_apart(cfg)
+
+
+@pytest.mark.parametrize("S", [1, 33, 100, 200])
+def test_one_block(S):
+    check_apart(synth._enc(2, 128, 2, 256, 32, 2, S, "bf16"))
