@@ -803,7 +803,7 @@ cudaError_t launch_fwd(FwdArgs p, cudaStream_t st) {
   auto k = R == 32 ? (sz == 0 ? adapter_fwd_mma_kernel<MB, MODE, 0, 2> : adapter_fwd_mma_kernel<MB, MODE, 1, 2>)
          : sz == 0 ? adapter_fwd_mma_kernel<MB, MODE, 0, 1>
          : sz == 1 ? adapter_fwd_mma_kernel<MB, MODE, 1, 1> : adapter_fwd_mma_kernel<MB, MODE, 2, 1>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(k, MAX_DYNAMIC_SMEM);
   if (e != cudaSuccess) return e;
   e = launch_pdl(k, dim3((p.T + R - 1) / R), dim3((p.H / COLS_PER_WARP) * 32), smem, st, p);
   note_launch(1);
@@ -818,7 +818,7 @@ cudaError_t launch_bwd(const BwdArgs& p, cudaStream_t st) {
   auto k = R == 32 ? (sz == 0 ? adapter_bwd_rows_mma_kernel<MB, 0, DH_F32, 2> : adapter_bwd_rows_mma_kernel<MB, 1, DH_F32, 2>)
          : sz == 0 ? adapter_bwd_rows_mma_kernel<MB, 0, DH_F32, 1>
          : sz == 1 ? adapter_bwd_rows_mma_kernel<MB, 1, DH_F32, 1> : adapter_bwd_rows_mma_kernel<MB, 2, DH_F32, 1>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(k, MAX_DYNAMIC_SMEM);
   if (e != cudaSuccess) return e;
   e = launch_pdl(k, dim3((p.T + R - 1) / R), dim3((p.H / COLS_PER_WARP) * 32), smem, st, p);
   note_launch(1);

@@ -30,7 +30,6 @@ namespace ra {
 namespace {
 
 constexpr int NW = 16, NT = NW * 32;
-constexpr int MAX_SMEM = 227 * 1024;
 
 template <typename T>
 __device__ __forceinline__ float4 ld4v(const T* p);
@@ -313,7 +312,7 @@ template <typename TX, typename TO, bool FWD, int TR, int TC>
 cudaError_t launch_rows(RowsArgs& p, cudaStream_t st) {
   auto k = adapter_rows_simt_kernel<TX, TO, FWD, TR, TC>;
   const size_t smem = (size_t)Plan<TX, TR, TC>(p.H, FWD && !p.f.no_norm).total;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(k, MAX_DYNAMIC_SMEM);
   if (e != cudaSuccess) return e;
   e = launch_pdl(k, dim3((p.T + 4 * TR - 1) / (4 * TR)), dim3(NT), smem, st, p);
   note_launch(1);
@@ -330,7 +329,7 @@ cudaError_t rows_dispatch(RowsArgs& p, cudaStream_t st) {
                      : tc == 8 ? (tr == 8 ? Plan<TX, 8, 8>(p.H, keep_v).total : tr == 4 ? Plan<TX, 4, 8>(p.H, keep_v).total
                                                                                         : Plan<TX, 2, 8>(p.H, keep_v).total)
                                : (tr == 4 ? Plan<TX, 4, 16>(p.H, keep_v).total : Plan<TX, 2, 16>(p.H, keep_v).total);
-    return smem <= MAX_SMEM;
+    return smem <= MAX_DYNAMIC_SMEM;
   };
   const int tc = p.m <= 32 ? 4 : p.m <= 64 ? 8 : 16, sms = device_sm_count();
   int tr = tc == 16 ? 4 : 8;

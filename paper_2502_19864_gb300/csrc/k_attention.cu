@@ -341,8 +341,9 @@ __global__ void __launch_bounds__(AT) attn_bwd_kernel(AttnArgs a) {
 
 template <typename T>
 cudaError_t fwd_impl(const AttnArgs& a, cudaStream_t st) {
-  const size_t smem = ((size_t)(RB + 2 * CB) * (a.head_dim + 4) + RB * LP) * sizeof(float);
-  cudaError_t e = cudaFuncSetAttribute(attn_fwd_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  auto bytes = [](int dh) { return ((size_t)(RB + 2 * CB) * (dh + 4) + RB * LP) * sizeof(float); };
+  const size_t smem = bytes(a.head_dim);
+  cudaError_t e = allow_smem(attn_fwd_kernel<T>, (int)bytes(MAXD));
   if (e != cudaSuccess) return e;
   e = launch_pdl(attn_fwd_kernel<T>, dim3((a.S + RB - 1) / RB, a.B * a.n_heads), dim3(AT), smem, st, a);
   note_launch(1);
@@ -368,8 +369,9 @@ cudaError_t bwd_impl(const AttnArgs& a, cudaStream_t st) {
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (attention_mma_ok(a)) return attention_bwd_mma(a, st);
-  const size_t smem = ((size_t)2 * (RB + CB) * (a.head_dim + 4) + 2 * RB * LP) * sizeof(float);
-  e = cudaFuncSetAttribute(attn_bwd_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  auto bytes = [](int dh) { return ((size_t)2 * (RB + CB) * (dh + 4) + 2 * RB * LP) * sizeof(float); };
+  const size_t smem = bytes(a.head_dim);
+  e = allow_smem(attn_bwd_kernel<T>, (int)bytes(MAXD));
   if (e != cudaSuccess) return e;
   e = launch_pdl(attn_bwd_kernel<T>, dim3((a.S + RB - 1) / RB, a.B * a.n_heads, 2), dim3(AT), smem, st, a);
   note_launch(1);

@@ -358,7 +358,7 @@ cudaError_t launch_simt(const GemmArgs& g, cudaStream_t st) {
   constexpr size_t ring = (size_t)NW * NS * (BT * LDA + (KN ? KC * BT : BT * LDA)) * sizeof(TI), part = (size_t)NW * BT * LDP * 4;
   constexpr size_t smem = ring > part ? ring : part;
   auto k = gemm_simt_kernel<TI, KN>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(k, (int)smem);
   if (e != cudaSuccess) return e;
   const int ks = ((g.K + NW - 1) / NW + KC - 1) / KC * KC;
   auto al = [](const void* p, int ld) { return ((uintptr_t)p & 15) == 0 && ld % 4 == 0; };
@@ -377,7 +377,7 @@ cudaError_t launch_simt(const GemmArgs& g, cudaStream_t st) {
       const int ns = std::min(kt / KT, tiles > device_sm_count() ? 3 : MAX_NS);
       const size_t sm = std::max((size_t)NW * ns * TSTAGE, part) + 1024;
       auto kern = split == 2 ? gemm_simt_tma_kernel<KN, 2> : gemm_simt_tma_kernel<KN, 1>;
-      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+      cudaError_t e = allow_smem(kern, (int)std::max((size_t)NW * MAX_NS * TSTAGE, part) + 1024);
       if (e != cudaSuccess) return e;
       cudaLaunchConfig_t cfg = {};
       cudaLaunchAttribute attr[2];

@@ -108,6 +108,16 @@ bool tma_map_bf16_batch(CUtensorMap* out, const void* ptr, int batch, int64_t ro
 bool tma_map_f32(CUtensorMap* out, const void* ptr, int64_t rows, int64_t cols, int64_t ld, int box_cols,
                  int box_rows);
 
+// Lets a kernel be launched with up to `bytes` of dynamic shared memory.  The limit belongs to the function and
+// not to the launch, and contexts on other threads launch the same kernels: so `bytes` is one constant for
+// all of a kernel's launches (its largest plan's), never the size of the launch at hand, which another
+// thread could lower between here and the launch.
+template <typename K>
+inline cudaError_t allow_smem(K* kernel, int bytes) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+constexpr int MAX_DYNAMIC_SMEM = 227 * 1024;  // of a CTA without static shared memory
+
 // ---------------------------------------------------------------------------------------
 // Attention (per (batch, head); token t = b*S + s; head hh at columns hh*dh of q/k/v).
 // ---------------------------------------------------------------------------------------

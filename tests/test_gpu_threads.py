@@ -1,0 +1,58 @@
+"""Contexts on their own host threads and streams: one context belongs to one thread at a time, but several
+contexts of other shapes may step at once.  The shapes differ in what they ask of the same kernels (dynamic
+shared memory among it), so a launch that goes by process-wide state fails or gives other results."""
+import threading
+
+import pytest
+
+import synth
+from paper_2502_19864_gb300 import ringada as R
+from gpu_helpers import GpuStepper
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    import __graft_entry__
+    __graft_entry__.build()
+
+
+@pytest.mark.parametrize("cfgs", [
+    (synth._enc(1, 64, 2, 64, 8, 2, 8, "f32"), synth._enc(1, 384, 3, 384, 16, 2, 40, "f32"),
+     synth._paper(1, 512, 16, 512, 16, 2, 24, "f32")),
+    (synth._enc(1, 256, 4, 256, 32, 2, 40, "bf16"), synth._enc(1, 768, 12, 768, 32, 2, 40, "bf16"),
+     synth._dec(1, 320, 5, 320, 40, 40, 2, 40, "bf16"))], ids=["f32", "bf16"])
+def test_contexts_of_other_shapes_at_once(cfgs, steps=400):
+    import torch
+    runs = [GpuStepper(cfg, synth.make_workload(cfg, 0)) for cfg in cfgs]
+    try:
+        alone = []
+        for run in runs:
+            run.step(1)
+            alone.append((run.logits.cpu(), run.model.grad(0, "WdF").cpu()))
+        torch.cuda.synchronize()
+        failed = []
+
+        def work(run, want):
+            try:
+                stream = torch.cuda.Stream()
+                for _ in range(steps):
+                    R.ra_forward(run.ctx, run.x.data_ptr(), run.labels.data_ptr(), run.cfg.batch, run.cfg.seq,
+                                 run.loss.data_ptr(), run.logits.data_ptr(), stream)
+                    R.ra_backward_truncated(run.ctx, run.cfg.n_layers - 1, stream)
+                R.ra_sync_status(run.ctx, stream)
+                if not (torch.equal(run.logits.cpu(), want[0]) and torch.equal(run.model.grad(0, "WdF").cpu(), want[1])):
+                    failed.append("%s: other results" % (run.cfg,))
+            except Exception as e:
+                failed.append("%s: %s" % (run.cfg, e))
+
+        threads = [threading.Thread(target=work, args=a) for a in zip(runs, alone)]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+        assert not failed, failed
+    finally:
+        for run in runs:
+            run.close()
