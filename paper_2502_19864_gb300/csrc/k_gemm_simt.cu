@@ -418,6 +418,22 @@ __global__ void swiglu_kernel(const void* gu, int ld_gu, int gu_dtype, void* h, 
 
 cudaError_t gemm_simt(const GemmArgs& g, cudaStream_t st) {
   if (g.M <= 0 || g.N <= 0) return cudaSuccess;
+  // a grid's y dimension holds 65535 row tiles; the rows past them are a product of their own
+  constexpr int ROWS = 65535 * BT;
+  if (g.M > ROWS) {
+    auto down = [](const void* p, int64_t ld, int dt) {
+      return p ? const_cast<char*>(static_cast<const char*>(p)) + ROWS * ld * (int64_t)dtype_size(dt) : nullptr;
+    };
+    GemmArgs head = g, rest = g;
+    head.M = ROWS;
+    rest.M = g.M - ROWS;
+    rest.A = down(g.A, g.lda, g.in_dtype);
+    rest.C = down(g.C, g.ldc, g.c_dtype);
+    rest.C2 = down(g.C2, g.ldc2, g.c2_dtype);
+    rest.aux = down(g.aux, g.ldaux, g.aux_dtype);
+    const cudaError_t e = gemm_simt(head, st);
+    return e != cudaSuccess ? e : gemm_simt(rest, st);
+  }
   cudaError_t e = g.in_dtype == DT_BF16 ? (g.b_kn ? launch_simt<bf16, true>(g, st) : launch_simt<bf16, false>(g, st))
                                         : (g.b_kn ? launch_simt<float, true>(g, st) : launch_simt<float, false>(g, st));
   if (e != cudaSuccess || g.epi != EPI_SWIGLU) return e;
