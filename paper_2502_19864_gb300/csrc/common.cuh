@@ -69,6 +69,12 @@ __device__ __forceinline__ float ex2_fast(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
+// the same with results below 2^-126 (a scaling on either side of the exponential)
+__device__ __forceinline__ float ex2_subnormal(float x) {
+  float y;
+  asm("ex2.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
 // GELU and GELU' of the GEMM epilogues, which evaluate them for every element of a large tile and
 // are paced by it.  Phi(-|x|) = erfc(|x| / sqrt 2) / 2 by Abramowitz & Stegun 7.1.26,
 //   erfc(z) = (a1 r + ... + a5 r^5) exp(-z^2), r = 1 / (1 + 0.3275911 z), |error| <= 1.5e-7,

@@ -667,7 +667,9 @@ __global__ void __launch_bounds__(256) span_head_dw_reduce_kernel(const float* p
 // with all of a thread's NV loads in flight, and stays in registers (packed as stored) through the
 // maximum, the sum and the two writes.  8192 rows of 32000 bf16 logits with logits_out (2.1 GB):
 // 370 us (the floor is 308; 453 with the label tested per logit and expf's denormal handling); reading the row from memory in each of three passes, two bytes at a time, took 716.
-template <typename T, int NV>
+// TAIL: a probability below 2^-126 keeps its gradient.  Without: bf16 gradients over 256 rows or more, where
+// p / T is then under half the least bf16 and rounds to zero either way.
+template <typename T, int NV, bool TAIL>
 __global__ void __launch_bounds__(512, 2) vocab_ce_kernel(T* logits, int ld, const int32_t* labels, int Tn,
     int V, float* row_loss, float* logits_out, bool out16, unsigned* err) {
   constexpr int VEC = 16 / sizeof(T);
@@ -722,8 +724,8 @@ __global__ void __launch_bounds__(512, 2) vocab_ce_kernel(T* logits, int ld, con
   mx = red[0][0];
 #pragma unroll
   for (int w = 1; w < 16; ++w) mx = fmaxf(mx, red[0][w]);
-  // (the special-function exponential: about 2 ulp, and below 2^-126 zero, against the dozen-odd
-  // instructions of expf per logit over a 32000-wide vocabulary)
+  // (the special-function exponential: about 2 ulp, against the dozen-odd instructions of expf per logit
+  // over a 32000-wide vocabulary; terms below 2^-126 add nothing to a sum that holds a 1)
   constexpr float kLog2e = 1.4426950408889634f;
   float se = 0.f;
 #pragma unroll
@@ -747,7 +749,10 @@ __global__ void __launch_bounds__(512, 2) vocab_ce_kernel(T* logits, int ld, con
     if (e >= nvec) continue;
     float p[VEC];
 #pragma unroll
-    for (int i = 0; i < VEC; ++i) p[i] = ex2_fast((value(r[n], i) - lse) * kLog2e);
+    for (int i = 0; i < VEC; ++i) {
+      const float x = (value(r[n], i) - lse) * kLog2e;
+      p[i] = TAIL ? ex2_subnormal(x) : ex2_fast(x);
+    }
     if (e == lvec) {
 #pragma unroll
       for (int i = 0; i < VEC; ++i)
@@ -1207,7 +1212,7 @@ namespace {
 // logits) are read once; other widths, strides and alignments take the three-pass kernel.  Plain
 // launches: started under the vocabulary GEMM's tail the step of two LLaMA-shaped blocks took 5750 us
 // instead of 5675.
-template <typename T>
+template <typename T, bool TAIL>
 void launch_vocab_ce(void* logits, int ld, const int32_t* labels, int Tn, int V, float* row_loss,
                      float* logits_out, unsigned* err, cudaStream_t st) {
   constexpr int VEC = 16 / sizeof(T);
@@ -1218,8 +1223,8 @@ void launch_vocab_ce(void* logits, int ld, const int32_t* labels, int Tn, int V,
     return;
   }
   const bool out16 = V % 4 == 0 && ((uintptr_t)logits_out & 15) == 0;
-  auto k = nv <= 1 ? vocab_ce_kernel<T, 1> : nv <= 2 ? vocab_ce_kernel<T, 2>
-         : nv <= 4 ? vocab_ce_kernel<T, 4> : vocab_ce_kernel<T, 8>;
+  auto k = nv <= 1 ? vocab_ce_kernel<T, 1, TAIL> : nv <= 2 ? vocab_ce_kernel<T, 2, TAIL>
+         : nv <= 4 ? vocab_ce_kernel<T, 4, TAIL> : vocab_ce_kernel<T, 8, TAIL>;
   k<<<Tn, 512, 0, st>>>(x, ld, labels, Tn, V, row_loss, logits_out, out16, err);
 }
 }  // namespace
@@ -1227,8 +1232,9 @@ void launch_vocab_ce(void* logits, int ld, const int32_t* labels, int Tn, int V,
 cudaError_t vocab_ce(void* logits, int dtype, int ld, const int32_t* labels, int T, int V,
                      float* row_loss, float* loss, float* logits_out, unsigned* err,
                      cudaStream_t st) {
-  if (dtype == DT_BF16) launch_vocab_ce<bf16>(logits, ld, labels, T, V, row_loss, logits_out, err, st);
-  else launch_vocab_ce<float>(logits, ld, labels, T, V, row_loss, logits_out, err, st);
+  auto launch = dtype != DT_BF16 ? launch_vocab_ce<float, true>
+                : T < 256        ? launch_vocab_ce<bf16, true> : launch_vocab_ce<bf16, false>;
+  launch(logits, ld, labels, T, V, row_loss, logits_out, err, st);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   (void)launch_pdl(mean_kernel, dim3(1), dim3(256), (size_t)0, st, row_loss, T, loss);
