@@ -65,17 +65,27 @@ struct BwdPlan {
 };
 
 // Rows [row, row + 128) of sequence b of a [B, S, columns] matrix, columns from col on, into a swizzled 128 x
-// DH block by TMA, one box per 64-wide atom.  Rows at or beyond S arrive as zeros: their probabilities are
-// zero, which times another sequence's values would not be zero where those are not finite.
-template <int DH>
-__device__ __forceinline__ void tma_block(const CUtensorMap* tm, uint32_t dst, uint64_t* bar, int col, int row, int b) {
+// DH block by TMA, one box per 64-wide atom.  Rows at or beyond S arrive as zeros (a 3-D map: columns, S, B):
+// their probabilities are zero, which times another sequence's values would not be zero where those are not
+// finite.  FLAT: S is a multiple of 128, there are no such rows and the map is 2-D (columns, B S).
+template <int DH, bool FLAT>
+__device__ __forceinline__ void tma_block(const CUtensorMap* tm, uint32_t dst, uint64_t* bar, int col, int row, int b,
+                                          int S) {
 #pragma unroll
-  for (int n = 0; n < DH / 64; ++n)
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst + n * (BR * 128)),
-        "l"(reinterpret_cast<uint64_t>(tm)), "r"(col + 64 * n), "r"(row), "r"(b), "r"(smem_u32(bar))
-        : "memory");
+  for (int n = 0; n < DH / 64; ++n) {
+    if constexpr (FLAT)
+      asm volatile(
+          "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+          " [%0], [%1, {%2, %3}], [%4];" ::"r"(dst + n * (BR * 128)),
+          "l"(reinterpret_cast<uint64_t>(tm)), "r"(col + 64 * n), "r"(b * S + row), "r"(smem_u32(bar))
+          : "memory");
+    else
+      asm volatile(
+          "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+          " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst + n * (BR * 128)),
+          "l"(reinterpret_cast<uint64_t>(tm)), "r"(col + 64 * n), "r"(row), "r"(b), "r"(smem_u32(bar))
+          : "memory");
+  }
 }
 // D[128 x 128] = A B^T over K = DH (both K-major 128 x DH blocks)
 template <int DH>
@@ -119,7 +129,7 @@ __device__ __forceinline__ void mma_xtb(uint32_t d, uint32_t x, uint32_t b) {
 // and at the end the shares change sides through the staging blocks and are added.  The scores, their
 // exponentials and dP are then computed once instead of in both passes, which set the pace: 32 x 16
 // heads of 256 76.9 us (92 in two passes), 32 x 12 of 128 22.7 (28.4).
-template <int DH, bool CAUSAL, bool ROPE, bool FUSED>
+template <int DH, bool CAUSAL, bool ROPE, bool FUSED, bool FLAT>
 __global__ void __launch_bounds__(NTHR, DH == 64 ? 2 : 1) attn_bwd_tc_kernel(const __grid_constant__ CUtensorMap tmQKV,
     const __grid_constant__ CUtensorMap tmDO, AttnArgs a) {
   using Pl = BwdPlan<DH>;
@@ -149,9 +159,9 @@ __global__ void __launch_bounds__(NTHR, DH == 64 ? 2 : 1) attn_bwd_tc_kernel(con
   constexpr uint32_t BLK_BYTES = BR * DH * 2;
   // q, k or v (part 0, 1, 2) rows of block blk_, or dO's, into a block of shared memory
   auto load_qkv = [&](uint32_t dst, int part, int blk_) {
-    tma_block<DH>(&tmQKV, dst, &load_bar, part * H + hh * DH, blk_ * BR, b);
+    tma_block<DH, FLAT>(&tmQKV, dst, &load_bar, part * H + hh * DH, blk_ * BR, b, S);
   };
-  auto load_do = [&](uint32_t dst, int blk_) { tma_block<DH>(&tmDO, dst, &load_bar, hh * DH, blk_ * BR, b); };
+  auto load_do = [&](uint32_t dst, int blk_) { tma_block<DH, FLAT>(&tmDO, dst, &load_bar, hh * DH, blk_ * BR, b, S); };
   if (warp == 1) {
     // this warp starts the first copies while warp 0 allocates TMEM (about 1200 cycles)
     if (elect_one()) {
@@ -486,9 +496,9 @@ __global__ void __launch_bounds__(NTHR, DH == 64 ? 2 : 1) attn_bwd_tc_kernel(con
   }
 }
 
-template <int DH, bool CAUSAL, bool ROPE, bool FUSED>
+template <int DH, bool CAUSAL, bool ROPE, bool FUSED, bool FLAT>
 cudaError_t launch_bwd_tc(const AttnArgs& a, cudaStream_t st) {
-  auto k = attn_bwd_tc_kernel<DH, CAUSAL, ROPE, FUSED>;
+  auto k = attn_bwd_tc_kernel<DH, CAUSAL, ROPE, FUSED, FLAT>;
   static bool attr_set = false;
   if (!attr_set) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdPlan<DH>::BYTES);
@@ -512,8 +522,9 @@ cudaError_t launch_bwd_tc(const AttnArgs& a, cudaStream_t st) {
   // qkv [B, S, 3 H] and dO [B, S, H] in boxes of 64 columns x 128 rows of one sequence
   const int H = a.n_heads * DH;
   CUtensorMap mq, md;
-  if (!tma_map_bf16_batch(&mq, a.qkv, a.B, a.S, 3LL * H, 3LL * H, 64, BR) ||
-      !tma_map_bf16_batch(&md, a.dO, a.B, a.S, H, H, 64, BR))
+  const int rows = FLAT ? a.B * a.S : a.S, batch = FLAT ? 0 : a.B;
+  if (!tma_map_bf16_batch(&mq, a.qkv, batch, rows, 3LL * H, 3LL * H, 64, BR) ||
+      !tma_map_bf16_batch(&md, a.dO, batch, rows, H, H, 64, BR))
     return cudaErrorNotSupported;
   cudaError_t e = cudaLaunchKernelEx(&cfg, k, mq, md, a);
   note_launch(1);
@@ -521,9 +532,14 @@ cudaError_t launch_bwd_tc(const AttnArgs& a, cudaStream_t st) {
 }
 template <int DH, bool CAUSAL, bool ROPE>
 cudaError_t dispatch_bwd_tc(const AttnArgs& a, cudaStream_t st) {
-  if constexpr (DH == 64)
-    if (a.S <= 2 * BR) return launch_bwd_tc<DH, CAUSAL, ROPE, true>(a, st);
-  return launch_bwd_tc<DH, CAUSAL, ROPE, false>(a, st);
+  if constexpr (DH == 64) {
+    if (a.S <= 2 * BR) return launch_bwd_tc<DH, CAUSAL, ROPE, true, false>(a, st);
+  } else {
+    // head dim 128 alone: 8 x 16 heads of 1024 (causal) take 442 us by the 2-D map and 460 by the 3-D one; the
+    // kernels for 64 and the forward take the same time by either (0.5 % at most)
+    if (a.S % BR == 0) return launch_bwd_tc<DH, CAUSAL, ROPE, false, true>(a, st);
+  }
+  return launch_bwd_tc<DH, CAUSAL, ROPE, false, false>(a, st);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -576,7 +592,7 @@ __global__ void __launch_bounds__(NTHR, 2) attn_fwd_blocks_tc_kernel(
   // q, k or v (part 0, 1, 2) rows of block blk_ into a block of shared memory; one lane calls it
   auto load = [&](uint32_t dst, uint64_t* lb, int part, int blk_) {
     mbar_expect_tx(lb, BR * DH * 2);
-    tma_block<DH>(&tmQKV, dst, lb, part * H + hh * DH, blk_ * BR, b);
+    tma_block<DH, false>(&tmQKV, dst, lb, part * H + hh * DH, blk_ * BR, b, S);
   };
   if (warp == 1) {
     // this warp starts the first copies while warp 0 allocates TMEM

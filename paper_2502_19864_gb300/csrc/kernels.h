@@ -101,7 +101,7 @@ int device_sm_count();
 bool tma_map_bf16(CUtensorMap* out, const void* ptr, int64_t rows, int64_t cols, int64_t ld, int box_cols,
                   int box_rows);
 // 3-D tensor map (columns, rows, batch) of `batch` such matrices one after the other: a box's rows past
-// the last of its own matrix arrive as zeros, not as the next one's
+// the last of its own matrix arrive as zeros, not as the next one's (batch 0: the 2-D map)
 bool tma_map_bf16_batch(CUtensorMap* out, const void* ptr, int batch, int64_t rows, int64_t cols, int64_t ld,
                         int box_cols, int box_rows);
 // the 2-D map for float32

@@ -18,8 +18,19 @@ def built():
 @pytest.mark.parametrize("S", [1, 128, 129, 256, 257])
 @pytest.mark.parametrize("decoder", [False, True])
 def test_block_edges(decoder, S):
-    cfg = (synth._dec(2, 128, 2, 128, 32, 40, 2, S, "bf16") if decoder else
-           synth._enc(2, 128, 2, 256, 32, 3, S, "bf16"))
+    check_every_depth(synth._dec(2, 128, 2, 128, 32, 40, 2, S, "bf16") if decoder else
+                      synth._enc(2, 128, 2, 256, 32, 3, S, "bf16"))
+
+
+@pytest.mark.parametrize("S", [127, 128, 256, 257])
+@pytest.mark.parametrize("decoder", [False, True])
+def test_head_dim_128(decoder, S):
+    """Two passes, with the copies of whole blocks (S a multiple of 128) and of blocks that a sequence ends in."""
+    check_every_depth(synth._dec(2, 256, 2, 128, 32, 40, 2, S, "bf16") if decoder else
+                      synth._span(2, 256, 2, 256, 32, 2, S, "bf16"))
+
+
+def check_every_depth(cfg):
     w = synth.make_workload(cfg, 0)
     ref = oracle_full(cfg, w)
     run = GpuStepper(cfg, w)
