@@ -76,41 +76,41 @@ __device__ __forceinline__ float ex2_subnormal(float x) {
   return y;
 }
 // GELU and GELU' of the GEMM epilogues, which evaluate them for every element of a large tile and
-// are paced by it.  Phi(-|x|) = erfc(|x| / sqrt 2) / 2 by Abramowitz & Stegun 7.1.26,
-//   erfc(z) = (a1 r + ... + a5 r^5) exp(-z^2), r = 1 / (1 + 0.3275911 z), |error| <= 1.5e-7,
-// with the halves folded into the coefficients: one reciprocal and one exponential per element (which
-// GELU' needs anyway) and 14 multiply-adds, where 7.1.28 and its four squarings took 25.  Against 64
-// bits over [-12, 12]: GELU 4.2e-7 at most and 0.7e-7 rms (7.6e-7 and 1.5e-7 by 7.1.28), GELU'
-// 3.0e-7 and 0.5e-7 (2.8e-7 and 0.7e-7); both leave the epilogue in bf16.
+// are paced by it.  Phi(-|x|) in the form of Abramowitz & Stegun 7.1.26,
+//   Phi(-|x|) = (b1 r + ... + b5 r^5) exp(-x^2 / 2), r = 1 / (1 + c |x|):
+// one reciprocal and one exponential per element (which GELU' needs anyway) and 14 multiply-adds, where
+// 7.1.28 and its four squarings took 25.  c and b are fitted for the least largest error, 5.9e-8; the published
+// ones give 7.5e-8, and as they are larger and of both signs they lose more to rounding near 0.  Largest (rms)
+// error against 64 bits over [-12, 12]: GELU 3.8e-7 (0.7e-7), by 7.1.28 8.8e-7 (1.7e-7); GELU' 2.3e-7
+// (0.3e-7), by 7.1.28 2.8e-7 (0.6e-7).  Both leave the epilogue in bf16.
 __device__ __forceinline__ float rcp_fast(float x) {
   float y;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-// Phi(x), and e = exp(-x^2 / 2)
+// Phi(x) up to its sign (1 - Phi(-x) for x >= 0, -Phi(x) below), and e = exp(-x^2 / 2)
 __device__ __forceinline__ float2 normal_cdf2(float2 x, float2& e) {
-  const float c = 0.3275911f * 0.70710678118654752f;
-  const float2 r = make_float2(rcp_fast(__fmaf_rn(fabsf(x.x), c, 1.0f)), rcp_fast(__fmaf_rn(fabsf(x.y), c, 1.0f)));
-  float2 p = __ffma2_rn(r, f2(0.5f * 1.061405429f), f2(0.5f * -1.453152027f));
-  p = __ffma2_rn(r, p, f2(0.5f * 1.421413741f));
-  p = __ffma2_rn(r, p, f2(0.5f * -0.284496736f));
-  p = __ffma2_rn(r, p, f2(0.5f * 0.254829592f));
-  p = __fmul2_rn(p, r);
+  const float2 r = make_float2(rcp_fast(__fmaf_rn(fabsf(x.x), 0.3308f, 1.0f)), rcp_fast(__fmaf_rn(fabsf(x.y), 0.3308f, 1.0f)));
+  float2 p = __ffma2_rn(r, f2(0.110379077f), f2(-0.375332892f));
+  p = __ffma2_rn(r, p, f2(0.0914756581f));
+  p = __ffma2_rn(r, p, f2(-0.204449788f));
+  p = __ffma2_rn(r, p, f2(-0.122071989f));
+  p = __fmul2_rn(p, r);  // minus the polynomial
   const float2 z = __fmul2_rn(__fmul2_rn(x, f2(-0.72134752044448170f)), x);  // -x^2 / 2 in powers of two
   e = make_float2(ex2_fast(z.x), ex2_fast(z.y));
-  const float2 lo = __fmul2_rn(p, e), hi = __ffma2_rn(lo, f2(-1.0f), f2(1.0f));
-  return make_float2(x.x < 0.f ? lo.x : hi.x, x.y < 0.f ? lo.y : hi.y);
+  return __ffma2_rn(p, e, make_float2(x.x < 0.f ? 0.f : 1.f, x.y < 0.f ? 0.f : 1.f));
 }
 __device__ __forceinline__ float2 gelu2(float2 x) {
   float2 e;
-  return __fmul2_rn(x, normal_cdf2(x, e));
+  const float2 Phi = normal_cdf2(x, e);
+  return make_float2(__fmul_rn(x.x, fabsf(Phi.x)), __fmul_rn(x.y, fabsf(Phi.y)));
 }
 // GELU(x) and GELU'(x) = Phi(x) + x phi(x) together
 __device__ __forceinline__ void gelu_both2(float2 x, float2& y, float2& dy) {
   float2 e;
-  const float2 Phi = normal_cdf2(x, e);
-  y = __fmul2_rn(x, Phi);
-  dy = __ffma2_rn(x, __fmul2_rn(e, f2(0.39894228040143268f)), Phi);
+  const float2 Phi = normal_cdf2(x, e), d = __fmul2_rn(__fmul2_rn(x, f2(0.39894228040143268f)), e);
+  y = make_float2(__fmul_rn(x.x, fabsf(Phi.x)), __fmul_rn(x.y, fabsf(Phi.y)));
+  dy = make_float2(__fadd_rn(d.x, fabsf(Phi.x)), __fadd_rn(d.y, fabsf(Phi.y)));
 }
 // SiLU and its derivative with the special-function exponential and the fast division (a few
 // ulp; they run per element in the SwiGLU epilogues).  For x below about -88 the denominator
