@@ -16,8 +16,6 @@
 // partial buffer would pass 64 KB) and sums the per-warp partials of z in a fixed order;
 // phase 2 gives each warp 64 of the H output columns; row statistics for the norm are
 // combined across warps in shared memory in a fixed order.
-#include <algorithm>
-
 #include "common.cuh"
 #include "kernels.h"
 
@@ -878,7 +876,7 @@ cudaError_t adapter_bwd_mma(const AdapterBwdArgs& a, const void* Wu_b, const voi
   d.dz = d.s + (size_t)a.T * a.m;
   d.partials = a.partials;
   // at most one wave of two CTAs an SM: 4096 x 768 on 12 x 26 CTAs left eight for a second wave
-  const int nchunk = std::max(1, std::min(adapter_dw_chunks(a.T, a.H), 2 * device_sm_count() / (a.H / DWC)));
+  const int nchunk = adapter_dw_chunks(a.T, a.H, a.H / DWC);
   d.chunk = (a.T + nchunk - 1) / nchunk;
   dim3 grid(a.H / DWC, nchunk);
   if (a.m == 32) e = launch_pdl(adapter_dw_mma_kernel<32>, grid, dim3(256), (size_t)0, st, d);

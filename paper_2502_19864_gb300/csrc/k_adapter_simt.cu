@@ -20,8 +20,6 @@
 // Measured (one row per warp pair and scalar loads before): 4608 x 768, m = 48, bf16 rows,
 // forward 485 -> 45 us, backward rows 240 -> 29 us; fp32 4096 x 768, m = 64, backward rows
 // 200 -> 33 us; fp32 128 x 128, m = 16, forward 31 -> 5.4 us.
-#include <algorithm>
-
 #include "common.cuh"
 #include "kernels.h"
 #include "simt.cuh"
@@ -441,10 +439,9 @@ cudaError_t adapter_bwd_simt(const AdapterBwdArgs& a, cudaStream_t st) {
   cudaError_t e = a.dh_dtype == DT_BF16 ? rows_dispatch<float, bf16, false>(p, st)
                                         : rows_dispatch<float, float, false>(p, st);
   if (e != cudaSuccess) return e;
-  // four CTAs an SM in one wave (608 in all; with a fifth on some SMs the launch takes a quarter longer),
-  // and no more chunks than the scratch is sized for; like that size a function of the shape alone
+  // four CTAs an SM in one wave (two products; with a fifth CTA on some SMs the launch takes a quarter longer)
   const int tiles = (a.H + DWI - 1) / DWI * ((a.m + DWJ - 1) / DWJ);
-  const int nchunk = std::max(1, std::min(adapter_dw_chunks(a.T, a.H), 304 / tiles));
+  const int nchunk = adapter_dw_chunks(a.T, a.H, tiles);
   const bool vm = a.m % 4 == 0 && al(a.z, 16) && al(a.dz, 16);
   const bool vh = a.H % 4 == 0 && al(a.g, 16) && al(a.h, 4 * dtype_size(a.dtype)) && al(a.partials, 16);
   const dim3 grid(tiles, nchunk, 2);

@@ -47,9 +47,8 @@ __global__ void adapter_dw_reduce_kernel(const float* partials, int nchunk, int 
   }
 }
 
-// Chunk count of the weight-gradient reduction: a pure function of (T, H), so the scratch
-// size planned on the host and the grid launched on any device agree, and the reduction
-// order (hence the bits of the result) does not depend on the device.
+// Most chunks of the weight-gradient reduction: a pure function of (T, H), so the scratch size planned on
+// the host and the grid launched on any device agree.
 constexpr int DW_COLS = 64, DW_ROWS = 16;
 constexpr int kDwTargetCtas = 304;
 int dw_chunks(int T, int H) {
@@ -1049,7 +1048,9 @@ size_t adapter_bwd_partials_floats(int T, int H, int m) {
   return (size_t)dw_chunks(T, H) * 2 * H * m;
 }
 
-int adapter_dw_chunks(int T, int H) { return dw_chunks(T, H); }
+int adapter_dw_chunks(int T, int H, int tiles) {
+  return max(1, min(dw_chunks(T, H), kDwTargetCtas / tiles));
+}
 
 cudaError_t adapter_dw_reduce(const float* partials, int nchunk, int H, int m, float* dWd,
                               float* dWu, cudaStream_t st) {

@@ -221,8 +221,10 @@ cudaError_t adapter_bwd(const AdapterBwdArgs& a, cudaStream_t st);
 cudaError_t adapter_bwd_mma(const AdapterBwdArgs& a, const void* Wu_b, const void* Wd_b,
                             cudaStream_t st);
 cudaError_t adapter_bwd_simt(const AdapterBwdArgs& a, cudaStream_t st);
-// chunk count of the dW reduction (a pure function of T and H) and its fixed-order sum
-int adapter_dw_chunks(int T, int H);
+// Row chunks of a dW reduction whose products have `tiles` output tiles, and the fixed-order sum over them: a
+// function of the shape alone, also where it keeps the launch to one wave of 304 tiles x chunks (two an SM on
+// 152 SMs), so that the order of the sums does not go by the device
+int adapter_dw_chunks(int T, int H, int tiles);
 cudaError_t adapter_dw_reduce(const float* partials, int nchunk, int H, int m, float* dWd,
                               float* dWu, cudaStream_t st);
 
