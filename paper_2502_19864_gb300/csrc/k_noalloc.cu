@@ -31,17 +31,16 @@ CUcontext g_scratch_ctx[kMaxDevices] = {};
 
 typedef CUresult (*CtxGetCurrentFn)(CUcontext*);
 CtxGetCurrentFn ctx_get_current() {
-  static CtxGetCurrentFn fn = nullptr;
-  static bool tried = false;
-  if (!tried) {
-    tried = true;
+  // (looked up in the initialiser: a second thread waits for the first one's answer)
+  static const CtxGetCurrentFn fn = []() -> CtxGetCurrentFn {
     void* p = nullptr;
     cudaDriverEntryPointQueryResult q;
     if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &p, 12000, cudaEnableDefault, &q) ==
             cudaSuccess &&
         q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<CtxGetCurrentFn>(p);
-  }
+      return reinterpret_cast<CtxGetCurrentFn>(p);
+    return nullptr;
+  }();
   return fn;
 }
 

@@ -1,6 +1,9 @@
 """Contexts on their own host threads and streams: one context belongs to one thread at a time, but several
 contexts of other shapes may step at once.  The shapes differ in what they ask of the same kernels (dynamic
 shared memory among it), so a launch that goes by process-wide state fails or gives other results."""
+import os
+import subprocess
+import sys
 import threading
 
 import pytest
@@ -56,3 +59,36 @@ def test_contexts_of_other_shapes_at_once(cfgs, steps=400):
     finally:
         for run in runs:
             run.close()
+
+
+FIRST_CALLS = """
+import sys, threading
+sys.path.insert(0, %r)
+import torch
+from paper_2502_19864_gb300 import ringada as R
+A, B = (torch.randn(256, 256, device="cuda").bfloat16() for _ in range(2))
+C = [torch.empty(256, 256, device="cuda") for _ in range(16)]
+R.lib(); torch.cuda.synchronize()
+at_once, failed = threading.Barrier(16), []
+def work(c):
+    torch.zeros(1, device="cuda")
+    at_once.wait()
+    try:
+        R.ra_gemm_bf16_epi(A.data_ptr(), B.data_ptr(), 256, 256, 256, R.RA_EPI_STORE, C_ptr=c.data_ptr(), c_dtype=R.RA_F32)
+    except Exception as e:
+        failed.append(str(e))
+threads = [threading.Thread(target=work, args=(c,)) for c in C]
+for t in threads: t.start()
+for t in threads: t.join()
+torch.cuda.synchronize()
+assert not failed, failed
+assert all(torch.equal(c, C[0]) for c in C)
+"""
+
+
+def test_first_calls_of_a_process_at_once():
+    """What is looked up once per process (a driver entry point, the device's kind) is there for every thread
+    that asks for it, also while another is still looking it up."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    for _ in range(3):
+        subprocess.run([sys.executable, "-c", FIRST_CALLS % root], check=True, timeout=300)
