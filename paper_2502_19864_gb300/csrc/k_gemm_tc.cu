@@ -995,10 +995,15 @@ bool make_map(CUtensorMap* out, const void* ptr, int64_t rows, int64_t cols, int
   cuuint64_t gstride[2] = {(cuuint64_t)ld * es, (cuuint64_t)(batch ? rows * ld : box_cols) * es};
   cuuint32_t box[3] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows, (cuuint32_t)(b3 ? blocks : 1)};
   cuuint32_t estride[3] = {1, 1, 1};
-  CUresult r = fn(out, dtype == DT_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
-                  b3 || batch ? 3 : 2, const_cast<void*>(ptr), gdim, gstride, box, estride,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  auto encode = [&] {
+    return fn(out, dtype == DT_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
+              b3 || batch ? 3 : 2, const_cast<void*>(ptr), gdim, gstride, box, estride,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  };
+  CUresult r = encode();
+  // a host thread that has made no CUDA runtime call has no context yet: one that does nothing gives it one
+  if (r == CUDA_ERROR_INVALID_CONTEXT && cudaFree(nullptr) == cudaSuccess) r = encode();
   if (r != CUDA_SUCCESS) return false;
   if (cache.size() > 4096) cache.clear();
   cache.emplace(key, *out);

@@ -92,3 +92,24 @@ def test_first_calls_of_a_process_at_once():
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     for _ in range(3):
         subprocess.run([sys.executable, "-c", FIRST_CALLS % root], check=True, timeout=300)
+
+
+def test_stand_alone_call_on_a_thread_new_to_cuda():
+    import torch
+    A, B = (torch.randn(128, 128, device="cuda").bfloat16() for _ in range(2))
+    C, failed = torch.empty(128, 128, device="cuda"), []
+    torch.cuda.synchronize()
+
+    def work():
+        try:
+            R.ra_gemm_bf16_epi(A.data_ptr(), B.data_ptr(), 128, 128, 128, R.RA_EPI_STORE, C_ptr=C.data_ptr(),
+                               c_dtype=R.RA_F32)
+        except Exception as e:
+            failed.append(str(e))
+
+    thread = threading.Thread(target=work)
+    thread.start()
+    thread.join()
+    assert not failed, failed
+    torch.cuda.synchronize()
+    assert (C.double() - A.double() @ B.double().T).abs().max().item() < 1e-4
