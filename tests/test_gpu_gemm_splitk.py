@@ -1,8 +1,11 @@
 """The split-K tcgen05 GEMM of few output tiles at its edges: one row, one k-block, K and N tails, a
-k-block more or less than the shares divide, one to eight CTAs to a tile, every epilogue, B as [N, K]
-and as stored [K, N]; against an fp32 matmul of the same bf16 operands, and bitwise repeatable."""
+k-block more or less than the shares divide, one to eight CTAs to a tile, every epilogue, B as [N, K] and as
+stored [K, N]; against a 64-bit matmul of the same bf16 operands, and bitwise repeatable (the gate|up
+epilogues through a decoder step)."""
 import pytest
 
+import synth
+from gpu_helpers import GpuStepper, check_step, oracle_full
 from paper_2502_19864_gb300 import ringada as R
 
 pytestmark = pytest.mark.gpu
@@ -63,3 +66,19 @@ def check_epilogues(M, N, K, kn):
 @pytest.mark.parametrize("M,N,K", SHAPES)
 def test_epilogues(M, N, K, kn):
     check_epilogues(M, N, K, kn)
+
+
+@pytest.mark.parametrize("H,heads,F,S", [(1024, 16, 2816, 120), (2048, 16, 512, 100), (2048, 16, 1024, 77),
+                                         (2112, 33, 2560, 33)])
+def test_gate_up_epilogues(H, heads, F, S):
+    """The gate|up epilogues through a decoder step: SwiGLU' on 64-wide tiles (H 1024: two CTAs to a tile; H
+    2048: eight) and SwiGLU on 128-wide ones (H 2048: eight and four CTAs to a tile; H 2112: two)."""
+    cfg = synth._dec(1, H, heads, F, 64, 96, 1, S, "bf16")
+    w = synth.make_workload(cfg, 0)
+    ref = oracle_full(cfg, w)
+    run = GpuStepper(cfg, w)
+    try:
+        loss = run.step(1)
+        check_step(cfg, loss, run.logits.double().cpu().numpy(), run.grads(0), run.head_grads(), ref, 0)
+    finally:
+        run.close()
