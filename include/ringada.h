@@ -248,7 +248,9 @@ ra_status ra_sync_status(ra_ctx* ctx, ra_stream_t stream);
 ra_status ra_selftest_wait_timeout(ra_ctx* ctx, int32_t limit_us, ra_stream_t stream);
 
 /* Diagnostic: y = f(x) for n float32 values with the activation code the step's kernels
- * use (the sigma of Eq. 1 and its derivative; SiLU of the decoder's SwiGLU FFN).
+ * use (the sigma of Eq. 1 and its derivative, as the adapters and the fp32 kernels evaluate
+ * it: the epilogues of the bf16 GEMMs have a form of their own, no further from the exact
+ * value; SiLU of the decoder's SwiGLU FFN).
  * which: 0 GELU(x) = x Phi(x), 1 GELU'(x) = Phi(x) + x phi(x), 2 SiLU, 3 SiLU'.
  * x_dev, y_dev: device arrays of n floats owned by the caller (may alias).  Enqueued on
  * `stream`; RA_ERR_ARG for another `which` or n < 0, RA_ERR_CUDA on a launch error. */

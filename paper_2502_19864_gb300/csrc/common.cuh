@@ -33,7 +33,7 @@ __device__ __forceinline__ float warp_max(float v) {
 //   erf(x) = 1 - (1 + a1 x + ... + a6 x^6)^-16 for x >= 0, odd extension, |error| <= 3e-7.
 // Evaluated without cancellation: with e = p - 1 carried exactly through the four squarings
 // (p^2k - 1 = e (2 + e)), erf = e16 / (1 + e16); x is clamped at 5, where erf is 1 in fp32.
-// Branch-free with one reciprocal.
+// Branch-free with one reciprocal.  Evaluated by the adapters and the fp32 kernels.
 __device__ __forceinline__ float erf_as7128(float x) {
   const float t = fminf(fabsf(x), 5.0f);
   float p = fmaf(t, 4.30638e-5f, 2.765672e-4f);

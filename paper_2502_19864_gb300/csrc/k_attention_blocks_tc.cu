@@ -20,7 +20,8 @@
 //   when causal):
 //     S = q_i k_j^T -> P (smem);  dP = dO_i v_j^T -> dS (smem, in place);  dQ_i += dS k_j
 // so dQ, dK and dV each accumulate in TMEM over the other index in a fixed order
-// (deterministic, no atomics).  P and dS are produced by the thread that owns their row, in
+// (deterministic, no atomics).  For head dim 64 and at most two blocks there are key passes alone, and dQ is
+// the sum of its one or two key blocks' shares (FUSED, below).  P and dS are produced by the thread that owns their row, in
 // the orientation the next product reads as its K-major A operand; the B operands of the
 // head-dim-wide products (dO_i, q_i, k_j) are read in place as MN-major blocks, one 64-wide
 // swizzle atom (and one MMA) per 64 head dims.  Rows and columns at or beyond S, and keys
@@ -218,8 +219,7 @@ __global__ void __launch_bounds__(NTHR, DH == 64 ? 2 : 1) attn_bwd_tc_kernel(con
     tc_fence_after();
     ok = ok && abort_sh == 0;
   };
-  // shared-memory writes by threads (and completed cp.async copies) -> visible to the
-  // tensor cores; then a barrier
+  // shared-memory writes by threads -> visible to the tensor cores; then a barrier
   auto publish = [&]() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     tc_fence_before();

@@ -172,8 +172,9 @@ __device__ __forceinline__ void finish(const GemmArgs& g, int ks, bool vc, bool 
 // lane holds 8 x 4 sums; each warp copies its own operands through a ring of three 8-deep chunks
 // (cp.async; the accumulation never waits for a whole load) and the warps' tiles are summed in warp
 // order.  Packed FMAs: two k at a time with B [N, K] (both operands come as pairs), two columns with
-// B [K, N].  Measured (64 x 64 tiles, one chain over K, scalar loads before): 128 x 128, K = 128 to 512:
-// 32 -> 6.8 us; 385 x 192, K = 192 to 768: 46 -> 8.8; 385 x 768, K = 192: 22.6 -> 10.4.
+// B [K, N].  A launch alone (64 x 64 tiles, one chain over K, scalar loads before): 128 x 128, K = 512 41 ->
+// 8.8 us, K = 128 14 -> 4.4; 385 x 192, K = 768 49 -> 11.5, K = 192 19 -> 5.3; 385 x 768, K = 192 22.7 -> 10.3.
+// The form for rows that TMA does not take; the one below serves the rest.
 template <typename TI, bool KN>
 __global__ void __launch_bounds__(NT, 2) gemm_simt_kernel(GemmArgs g, int ks, bool va, bool vb, bool vc) {
   constexpr int LDA = sizeof(TI) == 4 ? KC + 4 : KC;  // elements
@@ -246,8 +247,9 @@ __global__ void __launch_bounds__(NT, 2) gemm_simt_kernel(GemmArgs g, int ks, bo
 // touched 16 lines for 32 bytes of each, and starting the first two chunks took 1800 cycles (500 here).
 // What is left is the loop's shared-memory reads: a lane loads 12 floats per 32 multiply-adds, about 950
 // cycles for 8 k on one CTA an SM; so, where half the SMs have no tile and K is at least 512, a cluster
-// of two CTAs takes a half of K each.  128 x 128, K = 512: 8.4 -> 6.8 us; the fp32 tiny step 113 -> 105,
-// the 385-token fp32 step 405 -> 387.
+// of two CTAs takes a half of K each.  Against the form above, a launch alone: 128 x 128, K = 512 8.8 -> 6.9 us;
+// 385 x 192, K = 768 11.5 -> 10.8; at K below 256 0.4 us more alone, but in the stream the steps gain: the
+// fp32 tiny step 113 -> 105 us, the 385-token fp32 step 405 -> 387.
 constexpr int KT = 16, TSTAGE = BT * KT * 4 * 2, MAX_NS = 6;
 
 __device__ __forceinline__ void tma_box(const CUtensorMap* tm, uint32_t dst, uint64_t* bar, int c0, int c1) {

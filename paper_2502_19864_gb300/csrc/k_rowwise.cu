@@ -665,7 +665,8 @@ __global__ void __launch_bounds__(256) span_head_dw_reduce_kernel(const float* p
 // loss, and (logits_out) its logits in fp32.  Bound by HBM: the row is read once, 16 bytes a load
 // with all of a thread's NV loads in flight, and stays in registers (packed as stored) through the
 // maximum, the sum and the two writes.  8192 rows of 32000 bf16 logits with logits_out (2.1 GB):
-// 370 us (the floor is 308; 453 with the label tested per logit and expf's denormal handling); reading the row from memory in each of three passes, two bytes at a time, took 716.
+// 370 us (the floor is 308; 453 with the label tested per logit and expf's denormal handling); reading the row
+// from memory in each of three passes, two bytes at a time, took 716.
 // TAIL: a probability below 2^-126 keeps its gradient.  Without: bf16 gradients over 256 rows or more, where
 // p / T is then under half the least bf16 and rounds to zero either way.
 template <typename T, int NV, bool TAIL>

@@ -92,8 +92,8 @@ CONFIGS: Dict[str, ModelCfg] = {
     "small_paper_bf16": _paper(3, 256, 4, 1024, 32, 3, 100, "bf16"),
     # two 128-row key/query blocks with a ragged second block (S = 250)
     "small_enc_s250_bf16": _enc(2, 256, 4, 1024, 32, 2, 250, "bf16"),
-    # m = 64 and H = 512: the fused tcgen05 adapter forward over clusters of two CTAs, with a
-    # ragged last 128-row tile (T = 300), in both placements
+    # m = 64 and H = 512: the adapter kernels on 16-row CTAs of eight warps, with a ragged last one
+    # (T = 300), in both placements
     "small_enc_m64_bf16": _enc(2, 512, 8, 1024, 64, 3, 100, "bf16"),
     "small_paper_m64_bf16": _paper(2, 512, 8, 1024, 64, 3, 100, "bf16"),
     # the BERT-large layer shapes on 2 layers: its FFN-down and dX GEMMs run stream-K, on two

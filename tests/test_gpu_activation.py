@@ -1,8 +1,8 @@
 """The step's activation code (ra_eval_activation) against the exact functions in fp64.
 
-GELU and GELU' are evaluated in the kernels with erf from Abramowitz & Stegun formula
-7.1.28, whose published absolute error bound is 3e-7; evaluated in fp32 (without
-cancellation) it stays within 4.5e-7.  The bounds below carry that through
+GELU and GELU' are evaluated in the adapters and the fp32 kernels (the bf16 GEMMs' epilogues:
+test_gpu_epilogue_gelu.py) with erf from Abramowitz & Stegun formula 7.1.28, whose published absolute
+error bound is 3e-7; evaluated in fp32 (without cancellation) it stays within 4.5e-7.  The bounds below carry that through
 GELU(x) = x (1 + erf(x / sqrt 2)) / 2 and GELU'(x) = Phi(x) + x phi(x), plus fp32 rounding.
 SiLU and its derivative are checked at fp32 accuracy."""
 import numpy as np
