@@ -6,9 +6,10 @@
 //   backward  dz = (g W_up^T) GELU'(z); dh = g + dz W_down^T
 //   dW        per row-chunk partials of dW_up = GELU(z)^T g and dW_down^T = dz^T h
 //
-// Both row kernels are two skinny products per row tile, 4 T H m flops at 64 to 70 TFLOP/s of FFMA
-// against 12 to 16 T H bytes: bound by FFMA and its shared loads for m >= 32 or so, by latency for few rows.  One CTA of
-// 16 warps takes R = 4 TR rows:
+// Both row kernels are two skinny products per row tile, 4 T H m flops against 12 to 16 T H bytes.  No unit is at
+// its limit (4096 x 768, m = 64, backward rows: FFMA pipe 33 % and shared-memory path 30 % busy, an instruction
+// issued in 46 % of the cycles): the chain of copy, product and reduction of 16 warps an SM sets the time.
+// One CTA of 16 warps takes R = 4 TR rows:
 //   phase 1  [R, m] = X[R, H] W[H, m]: the warps split H; a lane holds TR x TC sums (4 lane rows
 //            x 8 lane columns, packed fp32x2 FMAs, which leave issue slots for the shared loads);
 //            the 16 partial tiles are summed in warp order;

@@ -246,7 +246,8 @@ __global__ void __launch_bounds__(NT, 2) gemm_simt_kernel(GemmArgs g, int ks, bo
 // of a warp's chunks are in flight at once where shared memory holds them.  By cp.async each instruction
 // touched 16 lines for 32 bytes of each, and starting the first two chunks took 1800 cycles (500 here).
 // What is left is the loop's shared-memory reads: a lane loads 12 floats per 32 multiply-adds, about 950
-// cycles for 8 k on one CTA an SM; so, where half the SMs have no tile and K is at least 512, a cluster
+// cycles for 8 k on one CTA an SM (385 x 192, K = 768 on 78 CTAs: the shared-memory path is busy for 54 % of
+// the cycles of an SM that has one); so, where half the SMs have no tile and K is at least 512, a cluster
 // of two CTAs takes a half of K each.  Against the form above, a launch alone: 128 x 128, K = 512 8.8 -> 6.9 us;
 // 385 x 192, K = 768 11.5 -> 10.8; at K below 256 0.4 us more alone, but in the stream the steps gain: the
 // fp32 tiny step 113 -> 105 us, the 385-token fp32 step 405 -> 387.
